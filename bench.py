@@ -42,17 +42,14 @@ WORKLOADS = {
            "over +-4 sigma_z each with its own 128x128 grid, 1e13 protons, the c2 ring, 216 SC kicks/turn"),
 }
 
-# FP64-pipe thread instructions per particle in kick_push_kernel (the turn
-# graph's variant), by segment content, from ncu's
+# The algorithm's float64 work per particle in kick_push_kernel, by segment
+# content, as the FP64-pipe thread instructions it takes when every map is
+# written in FP64 instructions: ncu's
 # sm__thread_inst_executed_pipe_fp64_pred_on per launch on the three segment
-# types of the bench ring (1e6 particles), fitted to the segments' element mix
-# (profiles/kick_push_c2.md gives the per-segment counts and the commands);
+# types of the bench ring (1e6 particles), of the build that did so
+# (profiles/kick_push_c2.md: 55.8, 68.0 and 18.0, mean 47.2 per particle-kick).
 # base = gather + kick + fused deposit.  The quadrupole reads its matrix
 # entries from the per-particle family cache (51.0 when it computes them).
-# The counts belong to the kernel sources whose SHA-256 (first 16 hex digits)
-# is FP64_INST_SOURCES_SHA (the three segment types measured on them: 55.8,
-# 68.0 and 18.0, mean 47.2 per particle-kick, the model's own figure); the
-# bench reports whether the sources still match.
 FP64_INST = {"base": 17.5, "drift": 12.2, "quad": 20.6, "sext": 5.0, "bend": 16.0, "rf": 30.0}
 FP64_INST_QUAD_UNCACHED = 51.0  # with the longitudinal kick (psigma changes at every kick: no cache); earlier build
 # split-TF32 form: float32 gather from the cached fixed-point weights
@@ -73,7 +70,7 @@ FP64_INST_LON_BEZIER_F32 = 13.95
 # cache; c2: mean of the three segment types), with the kernel sources'
 # SHA-256 (first 16 hex digits) they were captured on: the roofline's
 # "traffic" while the sources still match; other workloads report null.
-KP_TRAFFIC_TF32 = {"c2": (122.4e6, "741f33f43b3df3e1"),  # 1e6 particles (the working set partly stays in L2)
+KP_TRAFFIC_TF32 = {"c2": (127.3e6, "1daf2e920f0792b1"),  # 1e6 particles (the working set partly stays in L2)
                    "c4": (3860.0e6, "052c41cbfc714941"),  # 2.37e7 particles, batched (kick_push_traffic_c4_c5.md)
                    "c5": (1594.1e6, "052c41cbfc714941")}  # 1e7 particles in 32 slices
 # GB300: 152 SMs x 2 FP64 instructions per SM clock x 2.07 GHz maximum clock
@@ -84,8 +81,18 @@ FP64_PIPE_PEAK_TINST = 152 * 2 * 2.07e9 / 1e12
 # slice index two more)
 DEP_FP64_INST = 4.23
 DEP_FP64_INST_SLICE = 2.0
-KP_SOURCES = ("kick_push.cu", "maps.cuh", "cic.cuh", "fixpt.h", "sc_internal.cuh")
-FP64_INST_SOURCES_SHA = "741f33f43b3df3e1"
+# What the kernels of the tree issue to the FP64 pipe, measured the same way on
+# the sources whose SHA-256 (first 16 hex digits) is FP64_INST_SOURCES_SHA:
+# corrections and the path length in float pairs (csrc/dfloat.h).  By kernel
+# family: float64 fields; float32 fields with the series drift (split TF32, one
+# grid per bunch); float32 fields with the general drift (the other split forms).
+FP64_ISSUED = {
+    "f64": {"base": 17.34, "drift": 4.37, "quad": 6.33, "sext": 5, "bend": 16.0, "rf": 30.0},
+    "f32_series": {"base": 6.76, "drift": 3.2, "quad": 8.62, "sext": 5, "bend": 16.0, "rf": 30.0},
+    "f32": {"base": 6.76, "drift": 11.2, "quad": 8.62, "sext": 5, "bend": 16.0, "rf": 30.0},
+}
+KP_SOURCES = ("kick_push.cu", "maps.cuh", "cic.cuh", "fixpt.h", "dfloat.h", "sc_internal.cuh")
+FP64_INST_SOURCES_SHA = "1daf2e920f0792b1"
 # HBM bytes per particle-kick that the fused kick/push must move (algorithmic):
 # the six float64 coordinates read (48 B) and the five a kick and a push
 # change written back (40 B: psigma changes only in RF cavities); 96 B when
@@ -204,6 +211,14 @@ def element_mix(lat):
     mix = {name: int((t == code).sum()) for code, name in per.items()}
     mix["kicks"] = int((t == synth.MARK).sum())
     return mix
+
+
+def fp64_issued_per_kick(lat, precision, sliced):
+    """FP64-pipe instructions per particle-kick that the kernels of the tree issue."""
+    fam = "f64" if precision in ("fp64", "pipe_fp64") else "f32_series" if precision == "tf32x3" and not sliced else "f32"
+    t, mix = FP64_ISSUED[fam], element_mix(lat)
+    f = mix["kicks"] * (t["base"] + (FP64_INST_SLICE if sliced else 0.0))
+    return (f + sum(mix[k] * t[k] for k in ("drift", "quad", "sext", "bend", "rf"))) / mix["kicks"]
 
 
 def fp64_inst_per_turn(lat, precision):
@@ -694,7 +709,10 @@ def run_ours(args):
     W.trace(h, False)
     kp_avg_ms = kp_ms / traced
     inst_per_kick = inst_turn / n_kicks
-    achieved = inst_per_kick * n / (kp_avg_ms * 1e-3) / 1e12
+    issued = fp64_issued_per_kick(W.lat, args.precision, bool(getattr(W, "slices", None)))
+    if args.longitudinal or args.gather == "bezier":
+        issued = None  # not captured with these options: the algorithm's work alone
+    achieved = (issued or inst_per_kick) * n / (kp_avg_ms * 1e-3) / 1e12
     sha = kp_sources_sha()
     mix = element_mix(W.lat)
     rf = mix["rf"] > 0 or args.longitudinal
@@ -712,10 +730,12 @@ def run_ours(args):
                 "peak_source": None,  # after the live probe below
                 "avg_launch_ms": kp_avg_ms,
                 "fp64_inst_per_particle_kick": inst_per_kick,
+                "fp64_issued_per_particle_kick": issued,
                 "fp64_inst_model": {"per_element": dict(FP64_INST, base_split_form=FP64_INST_BASE_F32),
                                     "element_mix_per_turn": mix,
                                     "source": "ncu sm__thread_inst_executed_pipe_fp64_pred_on per launch, "
                                               "profiles/kick_push_c2.md",
+                                    "issued_per_element": FP64_ISSUED,
                                     "fitted_on_sources_sha": FP64_INST_SOURCES_SHA, "current_sources_sha": sha,
                                     "current": sha == FP64_INST_SOURCES_SHA},
                 "hbm": {"achieved": hbm_achieved, "peak": hbm_peak, "unit": "GB/s", "frac": hbm_achieved / hbm_peak,

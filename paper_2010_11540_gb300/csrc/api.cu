@@ -329,6 +329,7 @@ void set_kick(KPParams& P, const sc_grid* g, double kl, double gamma0) {
   P.E = g->E;
   P.E32 = (const float2*)g->E;
   P.field32 = g->field32;
+  P.series = series_drift(g);
   P.kl = kl;
   if (g->lon || g->gather == SC_GATHER_BEZIER) {
     P.phi = g->pipe.phi;         // float64 form
@@ -344,6 +345,7 @@ void set_kick(KPParams& P, const sc_grid* g, double kl, double gamma0) {
 // The cell cache a deposit writes follows the deposit grid's field precision.
 void set_deposit(KPParams& P, sc_grid* d) {
   P.field32 = d->field32;
+  P.series = series_drift(d);
   P.do_deposit = 1;
   P.gd = d->geom;
   P.Q = d->Q;
@@ -912,6 +914,7 @@ sc_status sc_track_turns(sc_grid* g, const sc_particles* p, const sc_beam* b, co
     T->prologue = base_params(p, b);
     T->prologue.psc = T->psc;
     T->prologue.psc_mode = 2;
+    T->prologue.series = series_drift(g);
     T->prologue.field32 = g->field32;  // every launch of the plan takes the grid's kernel family (and block size)
     with_qcache(T->prologue);
     if (!T->has_head && T->n_kicks > 0) {
@@ -962,6 +965,7 @@ sc_status sc_track_turns(sc_grid* g, const sc_particles* p, const sc_beam* b, co
     };
     auto launch = [&](KPParams P, bool dep) {
       P.field32 = g->field32;
+      P.series = series_drift(g);
       P.traversal = T->kp_trav;
       return launch_kick_push(P, dep ? g : nullptr, dep ? T->kp_blocks_dep : T->kp_blocks_plain, g->stream,
                               T->kp_threads);

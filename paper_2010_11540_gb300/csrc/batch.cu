@@ -178,7 +178,7 @@ template <class Capture, class Blocks>
 sc_status tune_batch_shape(sc_batch* B, BatchPlan* T, const sc_bunch* bunches, const std::vector<int64_t>& counts,
                            const std::vector<KPParams>& descs, Capture&& capture, Blocks&& set_blocks) {
   const int nb = B->n_bunches;
-  const bool f32 = split_solve(B->precision);
+  const bool f32 = split_solve(B->precision), series = series_drift(B->cls[0]);
   cudaStream_t S = B->stream;
   const int kicks = T->n_kicks < kShapeTuneKicks ? T->n_kicks : kShapeTuneKicks;
   int64_t total = 0;
@@ -298,7 +298,7 @@ sc_status tune_batch_shape(sc_batch* B, BatchPlan* T, const sc_bunch* bunches, c
         copy_bunches();
         clear_q();
         if (st == SC_OK)
-          st = launch_kick_push_batched(d_sdescs, d_blk, (int)bl.size(), T->tile_cells, f32, T->launch_cache[0] != 0,
+          st = launch_kick_push_batched(d_sdescs, d_blk, (int)bl.size(), T->tile_cells, f32, series, T->launch_cache[0] != 0,
                                         T->launch_xe[0] != 0, S, th);
         cu(cudaEventRecord(e0, S), "cudaEventRecord");
         cu(cudaGraphLaunch(exec, S), "cudaGraphLaunch(shape trial)");
@@ -528,7 +528,8 @@ sc_status sc_batch_track_turns(sc_batch* B, const sc_bunch* bunches, int n_turns
   put(&want_diag, sizeof want_diag);
   put(&B->trace, sizeof B->trace);
 
-  const bool f32 = split_solve(B->precision);
+  // (batch grids are unsliced and share one precision: one drift for all)
+  const bool f32 = split_solve(B->precision), series = series_drift(B->cls[0]);
   BatchPlan* T = B->plan;
   if (!T || T->key != key) {
     destroy_batch_plan(T);
@@ -707,7 +708,7 @@ sc_status sc_batch_track_turns(sc_batch* B, const sc_bunch* bunches, int n_turns
       const bool any = n_blocks > 0;  // some bunch holds particles
       if (T->has_head) {
         if (!cst && any)
-          cst = launch_kick_push_batched(d_descs + (size_t)L * nb, d_blocks, n_blocks, T->tile_cells, f32,
+          cst = launch_kick_push_batched(d_descs + (size_t)L * nb, d_blocks, n_blocks, T->tile_cells, f32, series,
                                          T->launch_cache[L] != 0, T->launch_xe[L] != 0, S, T->kp_threads);
         ++L;
       }
@@ -736,7 +737,7 @@ sc_status sc_batch_track_turns(sc_batch* B, const sc_bunch* bunches, int n_turns
         if (!cst && trace_on && cudaEventRecordWithFlags(T->ev[3 * k + 1], S, cudaEventRecordExternal) != cudaSuccess)
           cst = set_error(SC_ERR_CUDA, "event");
         if (!cst && any)
-          cst = launch_kick_push_batched(d_descs + (size_t)L * nb, d_blocks, n_blocks, T->tile_cells, f32,
+          cst = launch_kick_push_batched(d_descs + (size_t)L * nb, d_blocks, n_blocks, T->tile_cells, f32, series,
                                          T->launch_cache[L] != 0, T->launch_xe[L] != 0, S, T->kp_threads);
         if (!cst && trace_on && cudaEventRecordWithFlags(T->ev[3 * k + 2], S, cudaEventRecordExternal) != cudaSuccess)
           cst = set_error(SC_ERR_CUDA, "event");
@@ -818,7 +819,7 @@ sc_status sc_batch_track_turns(sc_batch* B, const sc_bunch* bunches, int n_turns
   if (T->n_blocks > 0) {
     if (!T->has_head && T->n_kicks > 0)
       for (sc_grid* g : B->cls) SC_CUDA(cudaMemsetAsync(g->Q, 0, cells_of(g) * g->nstack * 8, S));
-    if ((st = launch_kick_push_batched(T->d_descs, T->d_blocks, T->n_blocks, T->tile_cells, f32,
+    if ((st = launch_kick_push_batched(T->d_descs, T->d_blocks, T->n_blocks, T->tile_cells, f32, series,
                                        T->launch_cache[0] != 0, T->launch_xe[0] != 0, S, T->kp_threads)))
       return st;
   }

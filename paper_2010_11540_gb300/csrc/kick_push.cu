@@ -17,6 +17,9 @@ namespace sc {
 
 namespace {
 
+// A per-element constant as a float pair in a double's place; zero stays zero.
+double pack_f2(double v) { return f2_pack(v == 0.0 ? F2{0.f, 0.f} : f2_split(v)); }
+
 // Block sizes are multiples of 4 warps so that the four SM sub-partitions,
 // each with its own FP64 unit, carry the same number of warps.  Largest block
 // per variant (measured on the c2 workload): 768 threads (80 registers) for
@@ -71,11 +74,12 @@ __device__ __noinline__ void bezier_kick32(State& s, const KPParams& P, int cell
 }
 
 // The particle's coefficients of every quadrupole family, from its current ps
-// (k), into the cache.  Not inlined: it runs once per call and after RF cavities.
-__device__ __noinline__ void store_quad_cache(const KPParams& P, const PsConst& k, int64_t p) {
+// (ps and r of PsConst, passed by value: a reference would keep them in local
+// memory), into the cache.  Not inlined: it runs once per call and after RF cavities.
+__device__ __noinline__ void store_quad_cache(const KPParams& P, double ps, double r, int64_t p) {
   const size_t n = (size_t)P.n;
   for (int f = 0; f < P.qfam_n; ++f) {
-    const QuadCoef q = quad_coef(P.qfam[f], k);
+    const QuadCoef q = quad_coef(P.qfam[f], ps, r);
     double* c = P.qcache + (size_t)f * 6 * n + p;
     c[0] = q.cx;
     c[n] = q.sxa;
@@ -92,8 +96,9 @@ __device__ __noinline__ void store_quad_cache(const KPParams& P, const PsConst& 
 // the previous deposit is valid for the gather and is refreshed by this
 // deposit; F32: float32 fields and gather (the split-precision solve's fields
 // carry float32 accuracy; the fractions are then the deposit's own fixed-point
-// weights), else float64 fields and fractions.
-template <bool CACHE, bool F32, bool XE>
+// weights), else float64 fields and fractions; SERIES: the drift in float
+// pairs (map_drift, series_drift).
+template <bool CACHE, bool F32, bool XE, bool SERIES>
 __device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile, unsigned long long* tile,
                                                 int* tile_k, int64_t p_begin, int64_t p_end, int64_t p_step) {
   const int cells = P.gd.nx * P.gd.ny;
@@ -194,26 +199,28 @@ __device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile
     // the longitudinal kick changed psigma: its dependent quantities are recomputed and stored
     const bool fresh = psc_mode == 2 || (psc_mode == 1 && P.lon);
     if (psc_mode == 1 && !fresh) {
-      k.opd2 = P.psc[p];
-      k.opb = P.psc[n + p];
-      k.s1 = (P.psc_skip & 1) ? 0.0 : P.psc[2 * n + p];
+      k.d0 = P.psc[p];
+      k.d1 = P.psc[n + p];
+      k.eps = SERIES ? ((const float*)(P.psc + 2 * n))[p] : 0.f;
       k.r = (P.psc_skip & 1) ? 0.0 : P.psc[3 * n + p];
-      k.qi = (P.psc_skip & 2) ? 0.0 : P.psc[4 * n + p];
+      k.qi = f2_unpack((P.psc_skip & 2) ? 0.0 : P.psc[4 * n + p]);
     } else {
-      ps_const(k, s.ps, P.beta0_sq, fresh || P.has_quad != 0);
+      ps_const<SERIES>(k, s.ps, P.beta0_sq, fresh || P.has_quad != 0);
     }
     const bool quads = psc_mode != 0 || P.has_quad != 0;
     // the quadrupole coefficient cache holds this particle's values unless ps changed in this launch
     const double* qc = (P.qcache && psc_mode == 1 && !fresh) ? P.qcache + p : nullptr;
-    const bool changed = P.el ? push_elements<XE>(s, k, P.el, P.n_elem, P.beta0_sq, P.inv_gamma0_sq, quads, qc, n)
-                              : push_elements<XE>(s, k, P.inl, P.n_elem, P.beta0_sq, P.inv_gamma0_sq, quads, qc, n);
+    const double* psp = (P.ps_mode & 2) ? P.ps + p : nullptr;
+    const bool changed =
+        P.el ? push_elements<XE, SERIES>(s, k, P.el, P.n_elem, P.beta0_sq, P.inv_gamma0_sq, quads, qc, n, psp)
+             : push_elements<XE, SERIES>(s, k, P.inl, P.n_elem, P.beta0_sq, P.inv_gamma0_sq, quads, qc, n, psp);
     if (fresh || (psc_mode == 1 && changed)) {
-      P.psc[p] = k.opd2;
-      P.psc[n + p] = k.opb;
-      P.psc[2 * n + p] = k.s1;
+      P.psc[p] = k.d0;
+      P.psc[n + p] = k.d1;
+      if (SERIES) ((float*)(P.psc + 2 * n))[p] = k.eps;
       P.psc[3 * n + p] = k.r;
-      P.psc[4 * n + p] = k.qi;
-      if (P.qcache) store_quad_cache(P, k, p);
+      P.psc[4 * n + p] = f2_pack(k.qi);
+      if (P.qcache) store_quad_cache(P, s.ps, k.r, p);
     }
     if (P.do_deposit) {
       double fx = 0.0, fy = 0.0;
@@ -256,7 +263,7 @@ __device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile
 
 // One grid, one location.  TILE: the launch deposits (through the block's tile);
 // XE: thick sextupoles, exact dipoles or the Bezier gather may occur.
-template <bool TILE, bool CACHE, bool F32, bool XE>
+template <bool TILE, bool CACHE, bool F32, bool XE, bool SERIES>
 __global__ void __launch_bounds__(kp_max_threads<F32>()) kick_push_kernel(const __grid_constant__ KPParams P) {
   extern __shared__ unsigned long long tile[];
   __shared__ int tile_k;  // slice held by the tile (-1: not yet claimed)
@@ -278,14 +285,14 @@ __global__ void __launch_bounds__(kp_max_threads<F32>()) kick_push_kernel(const 
   const int64_t p_begin = chunked ? (int64_t)blockIdx.x * chunk : (int64_t)blockIdx.x * blockDim.x;
   const int64_t p_end = chunked ? min(P.n, (int64_t)(blockIdx.x + 1) * chunk) : P.n;
   const int64_t p_step = chunked ? (int64_t)blockDim.x : (int64_t)gridDim.x * blockDim.x;
-  kick_push_range<CACHE, F32, XE>(P, TILE, tile, &tile_k, p_begin, p_end, p_step);
+  kick_push_range<CACHE, F32, XE, SERIES>(P, TILE, tile, &tile_k, p_begin, p_end, p_step);
 }
 
 // Many bunches, one location each, one launch.  Block b works for bunch
 // blocks[b].x (its descriptor descs[bunch], copied to shared memory) on the
 // contiguous chunk blocks[b].y of blocks[b].z equal chunks of that bunch.
 // The bunch's deposit uses the tile when its grid's tile window fits tile_cells.
-template <bool CACHE, bool F32, bool XE>
+template <bool CACHE, bool F32, bool XE, bool SERIES>
 __global__ void __launch_bounds__(kpb_max_threads<F32>())
     kick_push_batched(const KPParams* __restrict__ descs, const int4* __restrict__ blocks, int tile_cells) {
   extern __shared__ unsigned long long tile[];
@@ -309,33 +316,48 @@ __global__ void __launch_bounds__(kpb_max_threads<F32>())
   const int64_t chunk = (sP.n + bt.z - 1) / bt.z;
   const int64_t p_begin = (int64_t)bt.y * chunk;
   const int64_t p_end = min(sP.n, p_begin + chunk);
-  kick_push_range<CACHE, F32, XE>(sP, use_tile, tile, &tile_k, p_begin, p_end, blockDim.x);
+  kick_push_range<CACHE, F32, XE, SERIES>(sP, use_tile, tile, &tile_k, p_begin, p_end, blockDim.x);
 }
 
 using KPKernel = void (*)(KPParams);
 using KPBatched = void (*)(const KPParams*, const int4*, int);
 
-// kick_push_kernel<TILE, CACHE, F32, XE> indexed by the four flags
-KPKernel kp_kernel(bool tile, bool cache, bool f32, bool xe) {
-  static const KPKernel k[16] = {
-      kick_push_kernel<false, false, false, false>, kick_push_kernel<false, false, false, true>,
-      kick_push_kernel<false, false, true, false>,  kick_push_kernel<false, false, true, true>,
-      kick_push_kernel<false, true, false, false>,  kick_push_kernel<false, true, false, true>,
-      kick_push_kernel<false, true, true, false>,   kick_push_kernel<false, true, true, true>,
-      kick_push_kernel<true, false, false, false>,  kick_push_kernel<true, false, false, true>,
-      kick_push_kernel<true, false, true, false>,   kick_push_kernel<true, false, true, true>,
-      kick_push_kernel<true, true, false, false>,   kick_push_kernel<true, true, false, true>,
-      kick_push_kernel<true, true, true, false>,    kick_push_kernel<true, true, true, true>};
-  return k[(tile ? 8 : 0) + (cache ? 4 : 0) + (f32 ? 2 : 0) + (xe ? 1 : 0)];
+// The kernels indexed by field type and drift (float64 fields always take the
+// series drift), then by the flags.
+enum : int { FK_F64 = 0, FK_F32 = 1, FK_F32_SERIES = 2, FK_COUNT = 3 };
+int family(const KPParams& P) { return !P.field32 ? FK_F64 : P.series ? FK_F32_SERIES : FK_F32; }
+
+template <bool F32, bool SERIES>
+KPKernel kp_of(bool tile, bool cache, bool xe) {
+  static const KPKernel k[8] = {
+      kick_push_kernel<false, false, F32, false, SERIES>, kick_push_kernel<false, false, F32, true, SERIES>,
+      kick_push_kernel<false, true, F32, false, SERIES>,  kick_push_kernel<false, true, F32, true, SERIES>,
+      kick_push_kernel<true, false, F32, false, SERIES>,  kick_push_kernel<true, false, F32, true, SERIES>,
+      kick_push_kernel<true, true, F32, false, SERIES>,   kick_push_kernel<true, true, F32, true, SERIES>};
+  return k[(tile ? 4 : 0) + (cache ? 2 : 0) + (xe ? 1 : 0)];
+}
+KPKernel kp_kernel(int fam, bool tile, bool cache, bool xe) {
+  return fam == FK_F64   ? kp_of<false, true>(tile, cache, xe)
+         : fam == FK_F32 ? kp_of<true, false>(tile, cache, xe)
+                         : kp_of<true, true>(tile, cache, xe);
 }
 
-KPBatched kp_batched(bool cache, bool f32, bool xe) {
-  static const KPBatched k[8] = {kick_push_batched<false, false, false>, kick_push_batched<false, false, true>,
-                                 kick_push_batched<false, true, false>,  kick_push_batched<false, true, true>,
-                                 kick_push_batched<true, false, false>,  kick_push_batched<true, false, true>,
-                                 kick_push_batched<true, true, false>,   kick_push_batched<true, true, true>};
-  return k[(cache ? 4 : 0) + (f32 ? 2 : 0) + (xe ? 1 : 0)];
+template <bool F32, bool SERIES>
+KPBatched kpb_of(bool cache, bool xe) {
+  static const KPBatched k[4] = {
+      kick_push_batched<false, F32, false, SERIES>, kick_push_batched<false, F32, true, SERIES>,
+      kick_push_batched<true, F32, false, SERIES>, kick_push_batched<true, F32, true, SERIES>};
+  return k[(cache ? 2 : 0) + (xe ? 1 : 0)];
 }
+KPBatched kp_batched(int fam, bool cache, bool xe) {
+  return fam == FK_F64   ? kpb_of<false, true>(cache, xe)
+         : fam == FK_F32 ? kpb_of<true, false>(cache, xe)
+                         : kpb_of<true, true>(cache, xe);
+}
+
+// The families a field type may take.
+int fam_first(bool f32) { return f32 ? FK_F32 : FK_F64; }
+int fam_last(bool f32) { return f32 ? FK_F32_SERIES : FK_F64; }
 
 // Resident blocks per SM of the smallest-occupancy variant for this tile size.
 int min_blocks(int smem, bool tile) {
@@ -343,13 +365,13 @@ int min_blocks(int smem, bool tile) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int best = 1 << 30;
-  for (int v = 0; v < 8; ++v) {
-    const bool cache = v & 4, f32 = v & 2, xe = v & 1;
-    const KPKernel k = kp_kernel(tile, cache, f32, xe);
+  for (int v = 0; v < 4 * FK_COUNT; ++v) {
+    const int fam = v >> 2;
+    const KPKernel k = kp_kernel(fam, tile, v & 2, v & 1);
     if (tile) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes);
     int per = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, f32 ? kp_max_threads<true>() : kp_max_threads<false>(),
-                                                  tile ? smem : 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &per, k, fam != FK_F64 ? kp_max_threads<true>() : kp_max_threads<false>(), tile ? smem : 0);
     best = per < best ? per : best;
   }
   return sms * (best < 1 ? 1 : best);
@@ -370,8 +392,8 @@ int kick_push_blocks_at(int smem_bytes, bool tile, bool f32, int threads) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int best = 1 << 30;
-  for (int v = 0; v < 4; ++v) {
-    const KPKernel k = kp_kernel(tile, v & 2, f32, v & 1);
+  for (int v = 4 * fam_first(f32); v < 4 * (fam_last(f32) + 1); ++v) {
+    const KPKernel k = kp_kernel(v >> 2, tile, v & 2, v & 1);
     if (tile) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes);
     int per = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads, tile ? smem_bytes : 0);
@@ -383,14 +405,13 @@ int kick_push_blocks_at(int smem_bytes, bool tile, bool f32, int threads) {
 sc_status launch_kick_push(const KPParams& P, const sc_grid* dep, int blocks, cudaStream_t s, int threads) {
   const bool tile = P.do_deposit && dep;
   const bool cache = P.cell != nullptr;
-  const bool f32 = P.field32 != 0;
   const bool xe = P.has_xe != 0 || P.bezier != 0;
   // default: the variant's largest block (measured: the extra warps outweigh a partly empty last round)
-  if (threads <= 0) threads = kick_push_max_threads(f32);
+  if (threads <= 0) threads = kick_push_max_threads(P.field32 != 0);
   const int64_t need = (P.n + threads - 1) / threads;
   if (need < blocks) blocks = (int)(need > 0 ? need : 1);
   const int smem = tile ? tile_bytes(dep) : 0;
-  SC_CUDA(launch_pdl(kp_kernel(tile, cache, f32, xe), dim3(blocks), dim3(threads), (size_t)smem, s, P));
+  SC_CUDA(launch_pdl(kp_kernel(family(P), tile, cache, xe), dim3(blocks), dim3(threads), (size_t)smem, s, P));
   return SC_OK;
 }
 
@@ -401,26 +422,38 @@ int kick_push_batched_resident(int smem_bytes, bool f32, bool cache, int threads
   int dev = 0, sms = 0, per = 1 << 30;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  for (int v = 0; v < 8; ++v) {
-    const KPBatched k = kp_batched(v & 4, v & 2, v & 1);
+  for (int v = 0; v < 4 * FK_COUNT; ++v) {
+    const KPBatched k = kp_batched(v >> 2, v & 2, v & 1);
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes);
   }
-  for (int xe = 0; xe < 2; ++xe) {
+  for (int v = 2 * fam_first(f32); v < 2 * (fam_last(f32) + 1); ++v) {
     int p = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, kp_batched(cache, f32, xe), threads, smem_bytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, kp_batched(v >> 1, cache, v & 1), threads, smem_bytes);
     per = p < per ? p : per;
   }
   return sms * (per < 1 ? 1 : per);
 }
 
 sc_status launch_kick_push_batched(const KPParams* descs, const int4* blocks, int n_blocks, int tile_cells, bool f32,
-                                   bool cache, bool xe, cudaStream_t s, int threads) {
+                                   bool series, bool cache, bool xe, cudaStream_t s, int threads) {
   // (the shared-memory limit was raised by kick_push_batched_resident, called before any launch)
   if (threads <= 0) threads = kick_push_batched_threads(f32);
-  SC_CUDA(launch_pdl(kp_batched(cache, f32, xe), dim3(n_blocks), dim3(threads), (size_t)tile_cells * 8, s, descs,
+  SC_CUDA(launch_pdl(kp_batched(!f32 ? FK_F64 : series ? FK_F32_SERIES : FK_F32, cache, xe), dim3(n_blocks), dim3(threads), (size_t)tile_cells * 8, s, descs,
                      blocks, tile_cells));
   return SC_OK;
 }
+
+// The series drift rounds the positions' last bit differently from the general
+// one.  Float64 fields follow such a change continuously.  Split-precision
+// solves do not: a changed bit of charge re-rolls their float32 (or bf16)
+// roundings, which moves the tracked state by 2.6e-10 (relative L2, one turn of
+// the 216-location ring, at most over 64^2..256^2 grids and 3e4..6e6 particles)
+// with TF32 on one grid per bunch, 1.1e-9 with BF16, 4.5e-8 in a pipe and up
+// to 1e-5 on sliced grids, whose slices carry 50 times the line density.  Only
+// the first is below 1e-9, so the others keep the general drift and with it
+// the bits of every position and momentum.  One turn, 1e6 particles on 128^2,
+// TF32: series 16.5 ms, general 21.1 ms (float64 fields: 24.2 ms with the series).
+bool series_drift(const sc_grid* g) { return !g->field32 || (g->precision == SC_SOLVE_TF32X3 && g->nz == 1); }
 
 // Per-element constants in float64 on the host (libm), in the layouts that
 // maps.cuh documents for each element type.
@@ -435,6 +468,7 @@ void compile_elements(const sc_element* in, int n, const sc_beam* b, DevElem* ou
     switch (e.type) {
       case SC_DRIFT:
         d.p[0] = e.length;
+        d.p[1] = pack_f2(e.length);
         break;
       case SC_QUAD: {
         d.p[0] = e.length;
@@ -454,6 +488,9 @@ void compile_elements(const sc_element* in, int n, const sc_beam* b, DevElem* ou
         d.p[6] = sqk;
         d.p[7] = 1.0 / sqk;
         d.p[8] = e.length * e.k1;
+        d.p[9] = pack_f2(d.p[0]);
+        d.p[10] = pack_f2(d.p[1]);
+        d.p[11] = pack_f2(d.p[8]);
         break;
       }
       case SC_SEXT:

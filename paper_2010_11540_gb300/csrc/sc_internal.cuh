@@ -79,7 +79,7 @@ constexpr int kTileBytes = 200 * 1024;
 struct DevElem {
   int type;
   int flags;
-  double p[9];
+  double p[12];
 };
 
 // Segments up to this many elements travel inside the launch parameters.
@@ -102,6 +102,7 @@ struct KPParams {
   int2* fix;       // fixed-point fractions (ax, ay) of the deposit (float32 fields)
   // float32 fields: E32 holds (Ex, Ey) as float2 and the gather runs in float32
   int field32;
+  int series;      // the drift in float pairs (series_drift); float64 fields always take it
   const float2* E32;
   // deposit
   int do_deposit;
@@ -115,8 +116,8 @@ struct KPParams {
   int n_elem;
   int has_quad;       // the segment holds an SC_QUAD
   int has_xe;         // the segment holds a thick SC_SEXT or an SC_EXACT_BEND
-  // Per-particle ps-dependent quantities, 5 arrays of n: (1+delta)^2,
-  // 1 + beta0^2 ps, sqrt(1-ps), 1/sqrt(1-ps), 1/(4(1-ps)).  psc_mode 0: none
+  // Per-particle ps-dependent quantities (PsConst in maps.cuh), 5 arrays of n:
+  // d0, d1, eps (the drift's; eps floats), 1/sqrt(1-ps), 1/(4(1-ps)) (float pair).  psc_mode 0: none
   // (computed in registers), 1: read (rewritten after an RF cavity), 2: compute and write.
   double* psc;
   int psc_mode;
@@ -127,9 +128,8 @@ struct KPParams {
   double* qcache;
   const DevElem* qfam;  // the families' compiled elements (device)
   int qfam_n;
-  // psc arrays the segment does not read (psc_mode 1): bit 0 sqrt(1-ps) and
-  // 1/sqrt(1-ps) (only quadrupoles computing their own matrix entries use
-  // them), bit 1 1/(4(1-ps)) (only thick quadrupoles)
+  // psc arrays the segment does not read (psc_mode 1): bit 0 1/sqrt(1-ps)
+  // (only quadrupoles computing their own matrix entries use it), bit 1 1/(4(1-ps)) (only thick quadrupoles)
   int psc_skip;
   // psigma traffic of the segment (psc_mode 1): bit 0 psigma is not changed
   // (no RF cavity, no longitudinal kick: not stored), bit 1 not read either
@@ -282,7 +282,9 @@ int kick_push_blocks_at(int smem_bytes, bool tile, bool f32, int threads);
 // deposits of grids whose tile window has at most tile_cells nodes go through the shared-memory tile.
 // threads: block size (0: the field type's largest, kick_push_batched_threads)
 sc_status launch_kick_push_batched(const KPParams* descs, const int4* blocks, int n_blocks, int tile_cells, bool f32,
-                                   bool cache, bool xe, cudaStream_t s, int threads = 0);
+                                   bool series, bool cache, bool xe, cudaStream_t s, int threads = 0);
+// which drift a grid's launches take (KPParams::series)
+bool series_drift(const sc_grid* g);
 int kick_push_batched_threads(bool f32);
 // resident blocks on the device at this block size (0: the largest)
 int kick_push_batched_resident(int smem_bytes, bool f32, bool cache, int threads = 0);
