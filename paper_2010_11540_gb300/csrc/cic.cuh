@@ -45,18 +45,57 @@ __device__ __forceinline__ int locate(const GridGeom& g, double x, double y, dou
   return locate<FRAC>(g, x, y, sg, a, fx, fy, k);
 }
 
+// A block's deposit tile in shared memory: the uint64 bins of its window as a
+// plane of low and a plane of high 32-bit words.  Shared memory has native
+// 32-bit atomic adds but only a compare-and-swap loop for 64 bits, so a bin is
+// added to by its low word, whose old value gives the carry, and its high word
+// (the sum is exact whatever the order of the adds).  Words of a plane lie
+// next to each other, so a warp's 32 random bins spread over all 32 banks.
+struct Tile {
+  uint32_t* lo;
+  uint32_t* hi;
+};
+__device__ __forceinline__ Tile tile_of(void* smem, const GridGeom& g) {
+  return Tile{(uint32_t*)smem, (uint32_t*)smem + g.wnx * g.wny};
+}
+
 // The four CIC weights in 2^-20 fixed point per axis: a (from locate), b =
 // 2^20 - a; the products sum to exactly 2^40 (32 x 32 -> 64-bit multiplies).
-// dst is either a shared-memory tile or the global grid (same [j][i] layout,
-// row length nx).
-__device__ __forceinline__ void deposit4(unsigned long long* dst, int nx, int cell, int2 a) {
+// q[0..3] = bx by, ax by, bx ay, ax ay.
+__device__ __forceinline__ void weights4(int2 a, unsigned long long (&w)[4]) {
   const unsigned ax = (unsigned)a.x, ay = (unsigned)a.y;
   const unsigned bx = 1048576u - ax, by = 1048576u - ay;
-  unsigned long long* q = dst + cell;
-  atomicAdd(q, (unsigned long long)bx * by);
-  atomicAdd(q + 1, (unsigned long long)ax * by);
-  atomicAdd(q + nx, (unsigned long long)bx * ay);
-  atomicAdd(q + nx + 1, (unsigned long long)ax * ay);
+  w[0] = (unsigned long long)bx * by;
+  w[1] = (unsigned long long)ax * by;
+  w[2] = (unsigned long long)bx * ay;
+  w[3] = (unsigned long long)ax * ay;
+}
+// Added to nodes (cell, cell + 1, cell + nx, cell + nx + 1) of the global
+// grid, or of a tile (same [j][i] layout, row length nx).
+__device__ __forceinline__ void add4(unsigned long long* Q, int nx, int cell, const unsigned long long (&w)[4]) {
+  unsigned long long* q = Q + cell;
+  atomicAdd(q, w[0]);
+  atomicAdd(q + 1, w[1]);
+  atomicAdd(q + nx, w[2]);
+  atomicAdd(q + nx + 1, w[3]);
+}
+__device__ __forceinline__ void add4(const Tile& t, int nx, int cell, const unsigned long long (&w)[4]) {
+  const int c[4] = {cell, cell + 1, cell + nx, cell + nx + 1};
+  uint32_t old[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) old[k] = atomicAdd(t.lo + c[k], (uint32_t)w[k]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t l = (uint32_t)w[k];
+    const uint32_t h = (uint32_t)(w[k] >> 32) + (old[k] + l < l ? 1u : 0u);
+    if (h) atomicAdd(t.hi + c[k], h);
+  }
+}
+template <class Dst>
+__device__ __forceinline__ void deposit4(const Dst& dst, int nx, int cell, int2 a) {
+  unsigned long long w[4];
+  weights4(a, w);
+  add4(dst, nx, cell, w);
 }
 
 // Deposit target of a particle in cell (i, j) of slice k (`cell` its global
@@ -89,7 +128,7 @@ __device__ __forceinline__ int deposit_key(bool use_tile, int* tile_k, const Gri
 }
 
 // The four CIC adds of one particle at its target key (deposit_key; -1: none).
-__device__ __forceinline__ void deposit_at(int key, int2 a, unsigned long long* tile, int wnx, unsigned long long* Q,
+__device__ __forceinline__ void deposit_at(int key, int2 a, const Tile& tile, int wnx, unsigned long long* Q,
                                            int nx) {
   if (key < 0) return;
   if (key & kGlobalKey)
@@ -109,7 +148,7 @@ __device__ __forceinline__ void deposit_at(int key, int2 a, unsigned long long* 
 // gets the same bits as with one atomic per weight.  When no two neighbouring
 // lanes share a key each lane adds its own.  (For particles in random order
 // the test itself costs more than it saves: callers use deposit_at there.)
-__device__ __forceinline__ void deposit_warp(unsigned mask, int key, int2 a, unsigned long long* tile, int wnx,
+__device__ __forceinline__ void deposit_warp(unsigned mask, int key, int2 a, const Tile& tile, int wnx,
                                              unsigned long long* Q, int nx) {
   const int lane = threadIdx.x & 31;
   const int prev = __shfl_up_sync(mask, key, 1);
@@ -142,15 +181,12 @@ __device__ __forceinline__ void deposit_warp(unsigned mask, int key, int2 a, uns
     const unsigned span = above ? ((1u << (__ffs(above) - 1)) - 1u) : 0xffffffffu;
     const unsigned long long n = (unsigned long long)__popc(mask & span & ~((1u << lane) - 1u));
     const unsigned long long one = 1048576ull;
-    const unsigned long long w11 = sxy, w10 = one * sx - sxy, w01 = one * sy - sxy;
-    const unsigned long long w00 = (n << 40) - one * ((unsigned long long)sx + sy) + sxy;
-    const bool global = key & kGlobalKey;
-    const int stride = global ? nx : wnx;
-    unsigned long long* q = global ? Q + (key & (kGlobalKey - 1)) : tile + key;
-    atomicAdd(q, w00);
-    atomicAdd(q + 1, w10);
-    atomicAdd(q + stride, w01);
-    atomicAdd(q + stride + 1, w11);
+    const unsigned long long w[4] = {(n << 40) - one * ((unsigned long long)sx + sy) + sxy, one * sx - sxy,
+                                     one * sy - sxy, sxy};
+    if (key & kGlobalKey)
+      add4(Q, nx, key & (kGlobalKey - 1), w);
+    else
+      add4(tile, wnx, key, w);
   }
 }
 
@@ -208,20 +244,22 @@ __device__ __forceinline__ void bezier_eval(const R* __restrict__ phi, int nx, i
   }
 }
 
-// Zero a shared-memory tile of `cells` int64 bins (whole block).
-__device__ __forceinline__ void tile_zero(unsigned long long* tile, int cells) {
-  for (int c = threadIdx.x; c < cells; c += blockDim.x) tile[c] = 0ull;
+// Zero a shared-memory tile of `cells` bins (whole block; 16-byte stores).
+__device__ __forceinline__ void tile_zero(void* tile, int cells) {
+  const int quads = cells >> 1;
+  for (int c = threadIdx.x; c < quads; c += blockDim.x) ((uint4*)tile)[c] = make_uint4(0u, 0u, 0u, 0u);
+  if ((cells & 1) && threadIdx.x == 0) ((unsigned long long*)tile)[cells - 1] = 0ull;
 }
 
 // Add the non-zero bins of a block's tile into the global grid Q (one
 // slice; whole block; caller synchronises before): bin (li, lj) of the window
 // is node (wx0 + li, wy0 + lj).  This is the only cross-block reduction of
 // the deposit.
-__device__ __forceinline__ void tile_flush(const unsigned long long* tile, unsigned long long* Q, const GridGeom& g) {
+__device__ __forceinline__ void tile_flush(const Tile& t, unsigned long long* Q, const GridGeom& g) {
   const int cells = g.wnx * g.wny;
   if (g.wnx == g.nx && g.wny == g.ny) {  // the tile is the whole slice: same indices
     for (int c = threadIdx.x; c < cells; c += blockDim.x) {
-      const unsigned long long v = tile[c];
+      const unsigned long long v = (unsigned long long)t.hi[c] << 32 | t.lo[c];
       if (v) atomicAdd(Q + c, v);
     }
     return;
@@ -230,7 +268,7 @@ __device__ __forceinline__ void tile_flush(const unsigned long long* tile, unsig
   int lj = threadIdx.x / g.wnx, li = threadIdx.x - lj * g.wnx;
   const int step_j = blockDim.x / g.wnx, step_i = blockDim.x - step_j * g.wnx;
   for (int c = threadIdx.x; c < cells; c += blockDim.x) {
-    const unsigned long long v = tile[c];
+    const unsigned long long v = (unsigned long long)t.hi[c] << 32 | t.lo[c];
     if (v) atomicAdd(Q + (size_t)(g.wy0 + lj) * g.nx + g.wx0 + li, v);
     lj += step_j;
     li += step_i;

@@ -23,10 +23,11 @@ __global__ void __launch_bounds__(kDepThreads) deposit_kernel(const double* __re
                                                                GridGeom g, unsigned long long* Q,
                                                                unsigned long long* n_out,
                                                                unsigned long long* n_nan) {
-  extern __shared__ unsigned long long tile[];
+  extern __shared__ uint4 tile_smem[];
+  const Tile tile = tile_of(tile_smem, g);
   __shared__ int tile_k;
   const int cells = g.nx * g.ny;
-  tile_zero(tile, g.wnx * g.wny);
+  tile_zero(tile_smem, g.wnx * g.wny);
   if (threadIdx.x == 0) tile_k = g.nz > 1 ? -1 : 0;
   __syncthreads();
   unsigned int out = 0, bad = 0;  // particles outside the grid; of those, non-finite ones

@@ -99,9 +99,10 @@ __device__ __noinline__ void store_quad_cache(const KPParams& P, double ps, doub
 // weights), else float64 fields and fractions; SERIES: the drift in float
 // pairs (map_drift, series_drift).
 template <bool CACHE, bool F32, bool XE, bool SERIES>
-__device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile, unsigned long long* tile,
+__device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile, void* tile_smem,
                                                 int* tile_k, int64_t p_begin, int64_t p_end, int64_t p_step) {
   const int cells = P.gd.nx * P.gd.ny;
+  const Tile tile = tile_of(tile_smem, P.gd);
   const int psc_mode = P.psc ? P.psc_mode : 0;
   const size_t n = (size_t)P.n;
   unsigned int out = 0;
@@ -265,10 +266,10 @@ __device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile
 // XE: thick sextupoles, exact dipoles or the Bezier gather may occur.
 template <bool TILE, bool CACHE, bool F32, bool XE, bool SERIES>
 __global__ void __launch_bounds__(kp_max_threads<F32>()) kick_push_kernel(const __grid_constant__ KPParams P) {
-  extern __shared__ unsigned long long tile[];
+  extern __shared__ uint4 tile_smem[];
   __shared__ int tile_k;  // slice held by the tile (-1: not yet claimed)
   if (TILE) {
-    tile_zero(tile, P.gd.wnx * P.gd.wny);
+    tile_zero(tile_smem, P.gd.wnx * P.gd.wny);
     if (threadIdx.x == 0) tile_k = P.gd.nz > 1 ? -1 : 0;
   }
   pdl_wait();  // fields, charge grid and particles of the previous kernels
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(kp_max_threads<F32>()) kick_push_kernel(const 
   const int64_t p_begin = chunked ? (int64_t)blockIdx.x * chunk : (int64_t)blockIdx.x * blockDim.x;
   const int64_t p_end = chunked ? min(P.n, (int64_t)(blockIdx.x + 1) * chunk) : P.n;
   const int64_t p_step = chunked ? (int64_t)blockDim.x : (int64_t)gridDim.x * blockDim.x;
-  kick_push_range<CACHE, F32, XE, SERIES>(P, TILE, tile, &tile_k, p_begin, p_end, p_step);
+  kick_push_range<CACHE, F32, XE, SERIES>(P, TILE, tile_smem, &tile_k, p_begin, p_end, p_step);
 }
 
 // Many bunches, one location each, one launch.  Block b works for bunch
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kp_max_threads<F32>()) kick_push_kernel(const 
 template <bool CACHE, bool F32, bool XE, bool SERIES>
 __global__ void __launch_bounds__(kpb_max_threads<F32>())
     kick_push_batched(const KPParams* __restrict__ descs, const int4* __restrict__ blocks, int tile_cells) {
-  extern __shared__ unsigned long long tile[];
+  extern __shared__ uint4 tile_smem[];
   __shared__ int tile_k;
   __shared__ KPParams sP;
   const int4 bt = blocks[blockIdx.x];
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(kpb_max_threads<F32>())
   __syncthreads();
   const bool use_tile = sP.do_deposit && sP.gd.wnx * sP.gd.wny <= tile_cells;
   if (use_tile) {
-    tile_zero(tile, sP.gd.wnx * sP.gd.wny);
+    tile_zero(tile_smem, sP.gd.wnx * sP.gd.wny);
     if (threadIdx.x == 0) tile_k = sP.gd.nz > 1 ? -1 : 0;
   }
   pdl_wait();
@@ -316,7 +317,7 @@ __global__ void __launch_bounds__(kpb_max_threads<F32>())
   const int64_t chunk = (sP.n + bt.z - 1) / bt.z;
   const int64_t p_begin = (int64_t)bt.y * chunk;
   const int64_t p_end = min(sP.n, p_begin + chunk);
-  kick_push_range<CACHE, F32, XE, SERIES>(sP, use_tile, tile, &tile_k, p_begin, p_end, blockDim.x);
+  kick_push_range<CACHE, F32, XE, SERIES>(sP, use_tile, tile_smem, &tile_k, p_begin, p_end, blockDim.x);
 }
 
 using KPKernel = void (*)(KPParams);
