@@ -128,4 +128,97 @@ SC_HD bool floor_index(double z, int limit, int& k) {
   return (unsigned)k < (unsigned)limit;
 }
 
+SC_HD uint64_t mulhi64(uint64_t a, uint64_t b) {
+#if defined(__CUDA_ARCH__)
+  return __umul64hi(a, b);
+#else
+  return (uint64_t)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+
+// One axis of a grid for fix_split: the coordinate as a 63-bit integer in
+// units of 2^-s, s set by the largest |x| of the grid, times inv_h as a 64-bit
+// integer gives xi with F fraction bits (F near 55), without an FP64
+// instruction.  That is nearer to (x - xmin) inv_h than the two rounded FP64
+// operations whose decision counts, and differs from them by at most T units:
+// only a coordinate within T of a place where the decision changes (a multiple
+// of 2^-21: weights change half-way between multiples of 2^-20, cells at
+// integers) is undecided, about one in 2^23.
+struct FixAxis {
+  uint64_t c;      // inv_h's significand, normalised to 2^63..2^64
+  uint64_t neg_x0; // minus (xmin 2^s less what T units of xi are)
+  uint64_t t;      // T
+  int32_t top;     // exponent field of the largest |x| of the grid; 0: not usable (fix_split is not called)
+  int32_t f;       // F
+  uint32_t near;   // 2 T in units of 2^-53 (rounded up)
+  int32_t limit;   // cells
+};
+
+// |(x - xmin) inv_h - its two-rounding value| <= cells 2^-52; the integers
+// truncate x (1 unit of D), xmin (1), the product (1) and T's own place (2).
+inline FixAxis make_fix_axis(double xmin, double inv_h, int cells) {
+  FixAxis a{};
+  a.limit = cells;
+  if (!(inv_h > 0.0) || cells < 1 || cells > 4096) return a;
+  const double xmax = xmin + cells / inv_h;
+  const double big = (xmin < 0 ? -xmin : xmin) > (xmax < 0 ? -xmax : xmax) ? (xmin < 0 ? -xmin : xmin) : (xmax < 0 ? -xmax : xmax);
+  const int top = (int)(f64_bits(big) >> 52), ei = (int)(f64_bits(inv_h) >> 52);
+  if (top < 100 || top > 1946 || ei < 100 || ei > 1946) return a;
+  const int s = 1084 - top, f = s + 1022 - ei;  // units of x; fraction bits of xi
+  if (f < 43 || f > 62) return a;               // (cells 2^f < 2^63 by construction)
+  a.c = ((f64_bits(inv_h) & ((1ull << 52) - 1)) | (1ull << 52)) << 11;
+  a.t = (uint64_t)((((unsigned __int128)(cells + 1) << f) >> 52) + 1) + 8;
+  // 2 T at most 2^-7 of the spacing of the places: else too many coordinates are undecided
+  if ((2 * a.t) >> (f - 28)) return a;
+  a.near = (uint32_t)(((unsigned __int128)(2 * a.t) << (85 - f)) >> 32) + 1;
+  // floor(xmin 2^s): xmin = m 2^(e - 1075), |xmin| 2^s = m 2^9 >> (top - e)
+  const uint64_t b = f64_bits(xmin);
+  const int e = (int)((b >> 52) & 0x7ff);
+  const uint64_t m = e ? (((b & ((1ull << 52) - 1)) | (1ull << 52)) << 9) : 0;
+  const int sh = top - e;
+  const uint64_t q = sh > 63 ? 0 : m >> sh;
+  const bool rest = sh > 63 ? xmin != 0.0 : (q << sh) != m;
+  int64_t x0 = (b >> 63) ? -(int64_t)q - (rest ? 1 : 0) : (int64_t)q;
+  const uint64_t off = (uint64_t)((((unsigned __int128)a.t) << 64) / a.c) + 1;  // T units of xi, in units of x
+  a.neg_x0 = (uint64_t)(-(x0 - (int64_t)off));
+  a.f = f;
+  a.top = top;
+  return a;
+}
+
+// Cell i, weight w (as cic_split's) and z = xi 2^F + T of coordinate x.
+// Returns 1: inside, as cic_split of the two-rounding xi says; 0: outside, as
+// it says; -1: undecided, ask cic_split.
+SC_HD int fix_split(const FixAxis& a, double x, int& i, int& w, uint64_t& z) {
+  const uint64_t b = f64_bits(x);
+  const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  const int sh = a.top - e;
+  // significand << 9 (62 bits), shifted to units of 2^-s
+  uint64_t m = (uint64_t)((((hi << 9) | (lo >> 23)) & 0x1fffffffu) | 0x20000000u) << 32 | (uint32_t)(lo << 9);
+#if defined(__CUDA_ARCH__)
+  asm("shr.b64 %0, %0, %1;" : "+l"(m) : "r"(sh));  // a shift beyond 63 gives 0
+#else
+  m = (sh < 0 || sh > 63) ? 0 : m >> sh;
+#endif
+  const uint64_t neg = (uint64_t)((int64_t)b >> 63);
+  z = mulhi64((m ^ neg) - neg + a.neg_x0, a.c);
+  i = (int)((uint32_t)(z >> 32) >> (a.f - 32));
+  w = (int)((((uint32_t)(z >> (a.f - 21)) - ((uint32_t)i << 21)) + 1u) >> 1);
+  if (sh < 0) return 0;  // beyond every node, infinite or NaN
+  if ((uint32_t)((z << (85 - a.f)) >> 32) < a.near) return -1;
+  return (uint32_t)i < (uint32_t)a.limit ? 1 : 0;
+}
+
+// The fraction xi - i of a decided coordinate, as a double (to 2^-52): its
+// bits under the exponent of 1, less 1 (one FP64 instruction).
+SC_HD double fix_fraction(const FixAxis& a, uint64_t z) {
+  const uint64_t fr = ((z - a.t) << (64 - a.f)) >> 12;
+#if defined(__CUDA_ARCH__)
+  return __dsub_rn(bits_f64(0x3ff0000000000000ull | fr), 1.0);
+#else
+  return bits_f64(0x3ff0000000000000ull | fr) - 1.0;
+#endif
+}
+
 }  // namespace sc

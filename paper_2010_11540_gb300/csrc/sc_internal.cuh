@@ -8,6 +8,7 @@
 #include <utility>
 #include <vector>
 
+#include "fixpt.h"
 #include "sc.h"
 
 namespace sc {
@@ -69,6 +70,9 @@ struct GridGeom {
   // slice, held in a block's shared memory (the whole slice when it fits in
   // kTileBytes, else the centred window that does)
   int wx0, wy0, wnx, wny;
+  // the axes in integers (x, y, and sigma when sliced); fix: all of them usable
+  FixAxis ax, ay, az;
+  int fix;
 };
 
 // Shared memory of a block's deposit tile (uint64 per node of its window).
