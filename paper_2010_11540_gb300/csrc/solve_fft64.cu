@@ -9,11 +9,16 @@
 // numbers as differencing phi, without the cancellation).  Dx is odd in x and
 // even in y, so its spectrum is i*Sx with Sx real; likewise Dy.
 //
-// Three kernels, each one FFT direction per block in shared memory
-// (Stockham radix-2, float64):
+// Three kernels, each one FFT direction per block in shared memory (Stockham
+// radix-2, float64; fft_smem.cuh):
 //   rows_fwd  : q row j (real, zero-padded)        -> F1[j][p], p = 0..nx
 //   columns   : F1[:, p] -> F(p, k) -> i Sx F, i Sy F -> inverse over k, keep j < ny
-//   rows_inv  : Hermitian half rows -> Ex, Ey at the nx x ny nodes.
+//   rows_inv  : Ex and Ey, both real, as real and imaginary part of one inverse transform.
+// The first stage of a transform of zero-padded data is a copy, those of the
+// inverse transforms are formed with the spectrum product or the symmetric
+// half on the way into shared memory, and the last stage forms only the half
+// that is kept.  The two inverse column transforms run side by side in two
+// halves of the block.
 #include <complex>
 #include <vector>
 
@@ -23,6 +28,7 @@ namespace sc {
 
 namespace {
 
+// blockDim.x = nx; block (row, stacked grid)
 __global__ void fft64_rows_fwd(const unsigned long long* __restrict__ Q, int nx, double scale,
                                const double* __restrict__ stack_scale,
                                double2* __restrict__ F1, const double2* __restrict__ twx) {
@@ -34,79 +40,84 @@ __global__ void fft64_rows_fwd(const unsigned long long* __restrict__ Q, int nx,
   double2 *a = sm, *b = sm + Mx;
   pdl_wait();
   if (stack_scale) scale = stack_scale[blockIdx.y];  // per stacked grid (bunches of a batch)
-  a[t] = make_double2((double)Q[(size_t)j * nx + t] * scale, 0.0);
-  a[t + nx] = make_double2(0.0, 0.0);
+  // first stage: the padding is zero, sum and difference are the datum itself
+  a[2 * t] = a[2 * t + 1] = make_double2((double)Q[(size_t)j * nx + t] * scale, 0.0);
   __syncthreads();
-  const double2* r = fft_smem<false>(a, b, Mx, twx);
+  const double2* r = fft_stages<false, false>(a, b, Mx, 2, t, twx);
   pdl_allow();
   for (int p = t; p <= nx; p += nx) F1[(size_t)j * (nx + 1) + p] = r[p];
 }
 
+// blockDim.x = 2 ny: threads t < ny the forward transform and the x field's
+// inverse one, the others the y field's; block (p, stacked grid)
 __global__ void fft64_columns(const double2* __restrict__ F1, int nx, int ny, const double* __restrict__ Sx,
                               const double* __restrict__ Sy, double2* __restrict__ Hx, double2* __restrict__ Hy,
                               const double2* __restrict__ twy, unsigned long long* Qzero) {
   extern __shared__ double2 sm[];
-  const int My = 2 * ny, p = blockIdx.x, t = threadIdx.x;
-  double2 *A = sm, *B = sm + My, *C = sm + 2 * My, *D = sm + 3 * My;
+  const int My = 2 * ny, p = blockIdx.x, f = threadIdx.x >= (unsigned)ny, t = threadIdx.x - f * ny;
+  double2 *A = sm, *B = sm + My, *C = sm + (2 + f) * My;
   const size_t so = (size_t)blockIdx.y * ny * (nx + 1);  // slice blockIdx.y
   F1 += so;
-  Hx += so;
-  Hy += so;
+  double2* H = (f ? Hy : Hx) + so;
+  const double* S = f ? Sy : Sx;
+  const double s0 = __ldg(S + (size_t)t * (nx + 1) + p), s1 = __ldg(S + (size_t)(t + ny) * (nx + 1) + p);
   pdl_wait();
   if (Qzero) {  // the row transform has read every slice's charge: clear it for the next deposit
     const int64_t total = (int64_t)gridDim.y * nx * ny;
-    for (int64_t c = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + t; c < total;
+    for (int64_t c = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; c < total;
          c += (int64_t)gridDim.x * gridDim.y * blockDim.x)
       Qzero[c] = 0ull;
   }
-  A[t] = F1[(size_t)t * (nx + 1) + p];
-  A[t + ny] = make_double2(0.0, 0.0);
+  // forward: stages 2 .. My/2 by the first half (the second keeps the barriers' count)
+  if (!f) A[2 * t] = A[2 * t + 1] = F1[(size_t)t * (nx + 1) + p];
   __syncthreads();
-  double2* R = fft_smem<false>(A, B, My, twy);
-  double2* freebuf = (R == A) ? B : A;
-  for (int k = t; k < My; k += ny) {
-    const double2 f = R[k];
-    const double sx = Sx[(size_t)k * (nx + 1) + p], sy = Sy[(size_t)k * (nx + 1) + p];
-    C[k] = make_double2(-sx * f.y, sx * f.x);
-    D[k] = make_double2(-sy * f.y, sy * f.x);
+  double2 *a = A, *b = B;
+  for (int Ns = 2; Ns < My; Ns <<= 1) {
+    if (!f) {
+      const int k = t & (Ns - 1), idx = ((t - k) << 1) + k;
+      double2 lo, hi;
+      fft_butterfly<false, false>(a[t], a[t + ny], k * (ny / Ns), My, twy, lo, hi);
+      b[idx] = lo;
+      b[idx + Ns] = hi;
+    }
+    __syncthreads();
+    double2* r = a;
+    a = b;
+    b = r;
   }
-  __syncthreads();
-  const double2* rx = fft_smem<true>(C, freebuf, My, twy);
-  const double2* ry = fft_smem<true>(D, R, My, twy);
+  // i S F and the inverse transform's first stage (no twiddles)
+  const double2 g0 = a[t], g1 = a[t + ny];
+  const double2 v0 = make_double2(-s0 * g0.y, s0 * g0.x), v1 = make_double2(-s1 * g1.y, s1 * g1.x);
+  C[2 * t] = make_double2(v0.x + v1.x, v0.y + v1.y);
+  C[2 * t + 1] = make_double2(v0.x - v1.x, v0.y - v1.y);
+  __syncthreads();  // (also: the forward result has been read, its buffers are free)
+  const double2* r = fft_stages<true, true>(C, f ? B : A, My, 2, t, twy);
   pdl_allow();
-  Hx[(size_t)t * (nx + 1) + p] = rx[t];
-  Hy[(size_t)t * (nx + 1) + p] = ry[t];
+  H[(size_t)t * (nx + 1) + p] = r[t];
 }
 
+// blockDim.x = nx; block (row, stacked grid)
 __global__ void fft64_rows_inv(const double2* __restrict__ Hx, const double2* __restrict__ Hy, int nx,
                                double inv_norm, double2* __restrict__ E, const double2* __restrict__ twx) {
   extern __shared__ double2 sm[];
   const int Mx = 2 * nx, j = blockIdx.x, t = threadIdx.x;
-  double2 *A = sm, *B = sm + Mx, *C = sm + 2 * Mx, *D = sm + 3 * Mx;
+  double2 *A = sm, *B = sm + Mx;
   const size_t so = (size_t)blockIdx.y * gridDim.x * (nx + 1);  // slice blockIdx.y
   E += (size_t)blockIdx.y * gridDim.x * nx;
   const double2* hx = Hx + so + (size_t)j * (nx + 1);
   const double2* hy = Hy + so + (size_t)j * (nx + 1);
   pdl_wait();
-  // p = t (<= nx) straight from the half spectrum; p = t + nx from Hermitian symmetry
-  A[t] = hx[t];
-  C[t] = hy[t];
-  {
-    const int pp = t + nx;
-    if (pp == nx) {
-      A[pp] = hx[nx];
-      C[pp] = hy[nx];
-    } else {
-      const double2 vx = hx[Mx - pp], vy = hy[Mx - pp];
-      A[pp] = make_double2(vx.x, -vx.y);
-      C[pp] = make_double2(vy.x, -vy.y);
-    }
-  }
+  // H = Hx + i Hy at p = t, and at p = t + nx from the Hermitian symmetry of each (p = nx itself is kept)
+  const double2 x0 = hx[t], y0 = hy[t];
+  const double2 v0 = make_double2(x0.x - y0.y, x0.y + y0.x);
+  const double2 x1 = hx[nx - t], y1 = hy[nx - t];
+  const double2 v1 = t == 0 ? make_double2(x1.x - y1.y, x1.y + y1.x) : make_double2(x1.x + y1.y, y1.x - x1.y);
+  A[2 * t] = make_double2(v0.x + v1.x, v0.y + v1.y);
+  A[2 * t + 1] = make_double2(v0.x - v1.x, v0.y - v1.y);
   __syncthreads();
-  const double2* rx = fft_smem<true>(A, B, Mx, twx);
-  const double2* ry = fft_smem<true>(C, D, Mx, twx);
+  const double2* r = fft_stages<true, true>(A, B, Mx, 2, t, twx);
   pdl_allow();
-  E[(size_t)j * nx + t] = make_double2(rx[t].x * inv_norm, ry[t].x * inv_norm);
+  E[(size_t)j * nx + t] = make_double2(r[t].x * inv_norm, r[t].y * inv_norm);
 }
 
 // Iterative radix-2 FFT on the host (used once per grid for the kernel spectra).
@@ -134,15 +145,6 @@ void host_fft(std::complex<double>* a, int n, int stride) {
 void host_fft2(std::vector<std::complex<double>>& a, int Mx, int My) {
   for (int b = 0; b < My; ++b) host_fft(a.data() + (size_t)b * Mx, Mx, 1);
   for (int c = 0; c < Mx; ++c) host_fft(a.data() + c, My, Mx);
-}
-
-std::vector<double2> twiddles(int M) {
-  std::vector<double2> t(M / 2);
-  for (int k = 0; k < M / 2; ++k) {
-    const double ang = -2.0 * M_PI * (double)k / (double)M;
-    t[k] = make_double2(std::cos(ang), std::sin(ang));
-  }
-  return t;
 }
 
 bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
@@ -199,7 +201,7 @@ sc_status fft64_create(sc_grid* g) {
       Sx[(size_t)k * (nx + 1) + p] = cx[(size_t)k * Mx + p].imag();
       Sy[(size_t)k * (nx + 1) + p] = cy[(size_t)k * Mx + p].imag();
     }
-  const auto twx = twiddles(Mx), twy = twiddles(My);
+  const auto twx = fft_twiddles(Mx), twy = fft_twiddles(My);
   const size_t half = (size_t)g->nstack * ny * (nx + 1) * sizeof(double2);  // one set per stacked grid
   if (cudaMalloc(&f.twx, twx.size() * sizeof(double2)) != cudaSuccess ||
       cudaMalloc(&f.twy, twy.size() * sizeof(double2)) != cudaSuccess || cudaMalloc(&f.F1, half) != cudaSuccess ||
@@ -241,10 +243,10 @@ sc_status fft64_solve(sc_grid* g, bool zero_q) {
   SC_CUDA(launch_pdl(fft64_rows_fwd, dim3(ny, nz), dim3(nx), 2 * Mx * sizeof(double2), g->stream,
                      (const unsigned long long*)g->Q, nx, scale, (const double*)g->stack_scale, f.F1,
                      (const double2*)f.twx));
-  SC_CUDA(launch_pdl(fft64_columns, dim3(nx + 1, nz), dim3(ny), 4 * My * sizeof(double2), g->stream,
+  SC_CUDA(launch_pdl(fft64_columns, dim3(nx + 1, nz), dim3(2 * ny), 4 * My * sizeof(double2), g->stream,
                      (const double2*)f.F1, nx, ny, (const double*)f.Sx, (const double*)f.Sy, f.Hx, f.Hy,
                      (const double2*)f.twy, zero_q ? g->Q : (unsigned long long*)nullptr));
-  SC_CUDA(launch_pdl(fft64_rows_inv, dim3(ny, nz), dim3(nx), 4 * Mx * sizeof(double2), g->stream, (const double2*)f.Hx,
+  SC_CUDA(launch_pdl(fft64_rows_inv, dim3(ny, nz), dim3(nx), 2 * Mx * sizeof(double2), g->stream, (const double2*)f.Hx,
                      (const double2*)f.Hy, nx, 1.0 / ((double)Mx * (double)My), g->E, (const double2*)f.twx));
   return SC_OK;
 }

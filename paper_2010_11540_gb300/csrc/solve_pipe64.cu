@@ -118,15 +118,6 @@ __global__ void pipe_fields(const double* __restrict__ phi, int nx, int ny, int 
   }
 }
 
-std::vector<double2> twiddles_p(int M) {
-  std::vector<double2> t(M / 2);
-  for (int k = 0; k < M / 2; ++k) {
-    const double ang = -2.0 * M_PI * (double)k / (double)M;
-    t[k] = make_double2(std::cos(ang), std::sin(ang));
-  }
-  return t;
-}
-
 bool pow2p(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
 }  // namespace
@@ -137,7 +128,7 @@ sc_status pipe_create(sc_grid* g) {
     return set_error(SC_ERR_UNSUPPORTED, "pipe solve needs nx - 1, ny - 1 powers of two in [8, 512]");
   PipePlan& f = g->pipe;
   const int Px = 2 * (nx - 1), Py = 2 * (ny - 1);
-  const auto twx = twiddles_p(Px), twy = twiddles_p(Py);
+  const auto twx = fft_twiddles(Px), twy = fft_twiddles(Py);
   // 1 / lambda_pq for q = 1..ny-2 (rows), p = 1..nx-2 (columns)
   std::vector<double> il((size_t)nx * ny, 0.0);
   for (int q = 1; q <= ny - 2; ++q)
