@@ -35,15 +35,17 @@ __device__ __forceinline__ void block_sums(double (&v)[C], double* __restrict__ 
   }
 }
 
-// The six means from the first pass's block sums, in a fixed order (every
-// caller gets the same bits).
-__device__ __forceinline__ void means_of(const double* __restrict__ partial, int n_blocks, int64_t n, double (&m)[6]) {
+// Column c of the block sums, summed by one warp: lane l takes rows l, l + 32,
+// ... and the lanes are added in a tree, a fixed order (every caller gets the
+// same bits).  One thread adding all 304 rows of six columns, as an earlier
+// form did in every block, waited 83 us for its chain of dependent loads and
+// adds (20,000 particles); a column's ten rows per lane are in flight together.
+__device__ __forceinline__ double column_sum(const double* __restrict__ partial, int n_blocks, int c) {
+  double v = 0.0;
+  for (int b = threadIdx.x & 31; b < n_blocks; b += 32) v += partial[(size_t)b * kNM + c];
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    double v = 0.0;
-    for (int b = 0; b < n_blocks; ++b) v += partial[(size_t)b * kNM + c];
-    m[c] = v / (double)n;
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
 // Pass 1: per-block sums of x, px, y, py, sigma, psigma -> partial[b][0..6).
@@ -76,11 +78,10 @@ __global__ void __launch_bounds__(kMomThreads) moments_central(const double* __r
                                                                const double* __restrict__ ps, int64_t n,
                                                                double* __restrict__ partial) {
   __shared__ double mean_s[6];
-  if (threadIdx.x == 0) {
-    double m[6];
-    means_of(partial, gridDim.x, n, m);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) mean_s[c] = m[c];
+  const int warp = threadIdx.x >> 5;
+  if (warp < 6) {
+    const double v = column_sum(partial, gridDim.x, warp) / (double)n;
+    if ((threadIdx.x & 31) == 0) mean_s[warp] = v;
   }
   __syncthreads();
   const double m0 = mean_s[0], m1 = mean_s[1], m2 = mean_s[2], m3 = mean_s[3], m4 = mean_s[4], m5 = mean_s[5];
@@ -100,22 +101,13 @@ __global__ void __launch_bounds__(kMomThreads) moments_central(const double* __r
   block_sums<8>(s, partial, 6);
 }
 
-// The 14 moments from both passes' block sums into out.
+// The 14 moments from both passes' block sums into out, one warp each.
+constexpr int kFinalThreads = 32 * kNM;
 __device__ __forceinline__ void moments_store(const double* __restrict__ partial, int n_blocks, int64_t n,
                                               double* out) {
-  __shared__ double tot[kNM];
-  if (threadIdx.x < kNM - 6) {
-    double v = 0.0;
-    for (int b = 0; b < n_blocks; ++b) v += partial[(size_t)b * kNM + 6 + threadIdx.x];
-    tot[6 + threadIdx.x] = v / (double)n;
-  }
-  if (threadIdx.x == 31) {
-    double m[6];
-    means_of(partial, n_blocks, n, m);
-    for (int c = 0; c < 6; ++c) tot[c] = m[c];
-  }
-  __syncthreads();
-  if (threadIdx.x < kNM) out[threadIdx.x] = tot[threadIdx.x];
+  const int c = threadIdx.x >> 5;
+  const double v = column_sum(partial, n_blocks, c) / (double)n;
+  if ((threadIdx.x & 31) == 0) out[c] = v;
 }
 
 // out = base_ptr[0] + stride * (*turn) receives the 14 moments; bumps *turn.
@@ -177,7 +169,7 @@ sc_status launch_moments(const sc_particles* p, double* partial, int n_blocks, d
                          int stride, cudaStream_t s) {
   moments_sums<<<n_blocks, kMomThreads, 0, s>>>(p->x, p->px, p->y, p->py, p->sigma, p->psigma, p->n, partial);
   moments_central<<<n_blocks, kMomThreads, 0, s>>>(p->x, p->px, p->y, p->py, p->sigma, p->psigma, p->n, partial);
-  moments_final<<<1, 32, 0, s>>>(partial, n_blocks, p->n, base_ptr, turn, stride);
+  moments_final<<<1, kFinalThreads, 0, s>>>(partial, n_blocks, p->n, base_ptr, turn, stride);
   SC_CUDA(cudaGetLastError());
   return SC_OK;
 }
@@ -283,7 +275,7 @@ extern "C" sc_status sc_moments_noalloc(const sc_particles* p, double* out, void
   cudaStream_t s = (cudaStream_t)stream;
   moments_sums<<<kMomBlocks, kMomThreads, 0, s>>>(p->x, p->px, p->y, p->py, p->sigma, p->psigma, p->n, scratch);
   moments_central<<<kMomBlocks, kMomThreads, 0, s>>>(p->x, p->px, p->y, p->py, p->sigma, p->psigma, p->n, scratch);
-  moments_final_to<<<1, 32, 0, s>>>(scratch, kMomBlocks, p->n, out);
+  moments_final_to<<<1, kFinalThreads, 0, s>>>(scratch, kMomBlocks, p->n, out);
   SC_CUDA(cudaGetLastError());
   return SC_OK;
 }
