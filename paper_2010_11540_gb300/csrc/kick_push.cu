@@ -76,7 +76,7 @@ __device__ __noinline__ void bezier_kick32(State& s, const KPParams& P, int cell
 // The particle's coefficients of every quadrupole family, from its current ps
 // (ps and r of PsConst, passed by value: a reference would keep them in local
 // memory), into the cache.  Not inlined: it runs once per call and after RF cavities.
-__device__ __noinline__ void store_quad_cache(const KPParams& P, double ps, double r, int64_t p) {
+__device__ __noinline__ void store_quad_cache(const KPParams& P, double ps, double r, uint32_t p) {
   const size_t n = (size_t)P.n;
   for (int f = 0; f < P.qfam_n; ++f) {
     const QuadCoef q = quad_coef(P.qfam[f], ps, r);
@@ -97,17 +97,32 @@ __device__ __noinline__ void store_quad_cache(const KPParams& P, double ps, doub
 // deposit; F32: float32 fields and gather (the split-precision solve's fields
 // carry float32 accuracy; the fractions are then the deposit's own fixed-point
 // weights), else float64 fields and fractions; SERIES: the drift in float
-// pairs (map_drift, series_drift).
+// pairs (map_drift, series_drift).  Indices are 32-bit (fewer than 2^24
+// particles): 64-bit ones cost another add per array access, 4% of a batch's turn.
 template <bool CACHE, bool F32, bool XE, bool SERIES>
 __device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile, void* tile_smem,
-                                                int* tile_k, int64_t p_begin, int64_t p_end, int64_t p_step) {
+                                                int* tile_k, uint32_t p_begin, uint32_t p_end, uint32_t p_step) {
   const int cells = P.gd.nx * P.gd.ny;
   const Tile tile = tile_of(tile_smem, P.gd);
   const int psc_mode = P.psc ? P.psc_mode : 0;
-  const size_t n = (size_t)P.n;
+  const uint32_t n = (uint32_t)P.n;
   unsigned int out = 0;
-  for (int64_t p = p_begin + threadIdx.x; p < p_end; p += p_step) {
+  for (uint32_t p = p_begin + threadIdx.x; p < p_end; p += p_step) {
     State s{P.x[p], P.px[p], P.y[p], P.py[p], P.sg[p], (P.ps_mode & 2) ? 0.0 : P.ps[p]};
+    PsConst k;
+    // the longitudinal kick changes psigma: its dependent quantities are recomputed and stored
+    const bool fresh = psc_mode == 2 || (psc_mode == 1 && P.lon);
+    auto load_psc = [&] {
+      k.d0 = P.psc[p];
+      k.d1 = P.psc[n + p];
+      k.eps = SERIES ? ((const float*)(P.psc + 2 * n))[p] : 0.f;
+      k.r = (P.psc_skip & 1) ? 0.0 : P.psc[3 * n + p];
+      k.qi = f2_unpack((P.psc_skip & 2) ? 0.0 : P.psc[4 * n + p]);
+    };
+    // loaded with the state where registers allow (float32 fields: 1.3% of a BF16 turn), else where first needed
+    // (early loads made the float64-field kernel 4% slower)
+    const bool kept = psc_mode == 1 && !fresh;
+    if (F32 && kept) load_psc();
     if (P.do_kick) {
       int cell;
       if (F32) {
@@ -196,18 +211,8 @@ __device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile
         }
       }
     }
-    PsConst k;
-    // the longitudinal kick changed psigma: its dependent quantities are recomputed and stored
-    const bool fresh = psc_mode == 2 || (psc_mode == 1 && P.lon);
-    if (psc_mode == 1 && !fresh) {
-      k.d0 = P.psc[p];
-      k.d1 = P.psc[n + p];
-      k.eps = SERIES ? ((const float*)(P.psc + 2 * n))[p] : 0.f;
-      k.r = (P.psc_skip & 1) ? 0.0 : P.psc[3 * n + p];
-      k.qi = f2_unpack((P.psc_skip & 2) ? 0.0 : P.psc[4 * n + p]);
-    } else {
-      ps_const<SERIES>(k, s.ps, P.beta0_sq, fresh || P.has_quad != 0);
-    }
+    if (!F32 && kept) load_psc();
+    if (!kept) ps_const<SERIES>(k, s.ps, P.beta0_sq, fresh || P.has_quad != 0);
     const bool quads = psc_mode != 0 || P.has_quad != 0;
     // the quadrupole coefficient cache holds this particle's values unless ps changed in this launch
     const double* qc = (P.qcache && psc_mode == 1 && !fresh) ? P.qcache + p : nullptr;
@@ -403,15 +408,28 @@ int kick_push_blocks_at(int smem_bytes, bool tile, bool f32, int threads) {
   return sms * (best < 1 ? 1 : best);
 }
 
+// Block size of a launch that leaves it open: the largest block, whose extra
+// warps outweigh a partly empty last round, or 384 threads when the bunch
+// would fill few SMs with largest blocks.  The line lies where twice the SMs
+// at work no longer pay for twice the tiles to clear and flush: n = 192 per SM,
+// or 384 with tiles up to 32 KB (measured per location, 2e4 particles: 64^2
+// 25.5 -> 22.6 us, 128^2 28.1 -> 27.6, 256^2 68.5 -> 66.9; 5e4: 64^2 25.6 ->
+// 23.2, but 256^2 68.8 -> 86.4; 1e5: 64^2 26.1 -> 26.3).
+int default_threads(int64_t n, bool f32, int smem) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return n <= (int64_t)sms * (smem <= 32 * 1024 ? 384 : 192) ? 384 : kick_push_max_threads(f32);
+}
+
 sc_status launch_kick_push(const KPParams& P, const sc_grid* dep, int blocks, cudaStream_t s, int threads) {
   const bool tile = P.do_deposit && dep;
   const bool cache = P.cell != nullptr;
   const bool xe = P.has_xe != 0 || P.bezier != 0;
-  // default: the variant's largest block (measured: the extra warps outweigh a partly empty last round)
-  if (threads <= 0) threads = kick_push_max_threads(P.field32 != 0);
+  const int smem = tile ? tile_bytes(dep) : 0;
+  if (threads <= 0) threads = default_threads(P.n, P.field32 != 0, smem);
   const int64_t need = (P.n + threads - 1) / threads;
   if (need < blocks) blocks = (int)(need > 0 ? need : 1);
-  const int smem = tile ? tile_bytes(dep) : 0;
   SC_CUDA(launch_pdl(kp_kernel(family(P), tile, cache, xe), dim3(blocks), dim3(threads), (size_t)smem, s, P));
   return SC_OK;
 }
