@@ -70,7 +70,7 @@ FP64_INST_LON_BEZIER_F32 = 13.95
 # cache; c2: mean of the three segment types), with the kernel sources'
 # SHA-256 (first 16 hex digits) they were captured on: the roofline's
 # "traffic" while the sources still match; other workloads report null.
-KP_TRAFFIC_TF32 = {"c2": (127.4e6, "70b1372c90210bd9"),  # 1e6 particles (the working set partly stays in L2)
+KP_TRAFFIC_TF32 = {"c2": (127.4e6, "1068f9b71ac01572"),  # 1e6 particles (the working set partly stays in L2)
                    "c4": (3860.0e6, "052c41cbfc714941"),  # 2.37e7 particles, batched (kick_push_traffic_c4_c5.md)
                    "c5": (1594.1e6, "052c41cbfc714941")}  # 1e7 particles in 32 slices
 # GB300: 152 SMs x 2 FP64 instructions per SM clock x 2.07 GHz maximum clock
@@ -87,12 +87,12 @@ DEP_FP64_INST_SLICE = 2.0
 # family: float64 fields; float32 fields with the series drift (split TF32, one
 # grid per bunch); float32 fields with the general drift (the other split forms).
 FP64_ISSUED = {
-    "f64": {"base": 15.34, "drift": 4.37, "quad": 6.33, "sext": 5, "bend": 16.0, "rf": 30.0},
+    "f64": {"base": 9.81, "drift": 3.98, "quad": 7.09, "sext": 5, "bend": 16.0, "rf": 30.0},
     "f32_series": {"base": 2.76, "drift": 3.2, "quad": 8.62, "sext": 5, "bend": 16.0, "rf": 30.0},
     "f32": {"base": 2.76, "drift": 11.2, "quad": 8.61, "sext": 5, "bend": 16.0, "rf": 30.0},
 }
 KP_SOURCES = ("kick_push.cu", "maps.cuh", "cic.cuh", "fixpt.h", "dfloat.h", "sc_internal.cuh")
-FP64_INST_SOURCES_SHA = "70b1372c90210bd9"
+FP64_INST_SOURCES_SHA = "1068f9b71ac01572"
 # HBM bytes per particle-kick that the fused kick/push must move (algorithmic):
 # the six float64 coordinates read (48 B) and the five a kick and a push
 # change written back (40 B: psigma changes only in RF cavities); 96 B when

@@ -327,6 +327,7 @@ void set_kick(KPParams& P, const sc_grid* g, double kl, double gamma0) {
   P.do_kick = (kl != 0.0);
   P.gk = g->geom;
   P.E = g->E;
+  P.dE = g->dE;
   P.E32 = (const float2*)g->E;
   P.field32 = g->field32;
   P.series = series_drift(g);
@@ -465,6 +466,14 @@ sc_status create_grid(sc_grid** out, int nx, int ny, double xmin, double xmax, d
   }
   cudaMemsetAsync(g->Q, 0, cells * 8, g->stream);
   cudaMemsetAsync(g->E, 0, cells * sizeof(double2), g->stream);
+  if (!g->field32) {
+    if ((e = cudaMalloc(&g->dE, cells * sizeof(double2))) != cudaSuccess) {
+      st = cuda_error(e, "cudaMalloc(grid)");
+      sc_destroy_grid(g);
+      return st;
+    }
+    cudaMemsetAsync(g->dE, 0, cells * sizeof(double2), g->stream);
+  }
   g->n_nan = g->n_out + nstack;
   cudaMemsetAsync(g->n_out, 0, 8 * (size_t)(nstack + 1), g->stream);
   g->dep_blocks = deposit_blocks_for(tile_bytes(g));
@@ -520,6 +529,7 @@ sc_status sc_destroy_grid(sc_grid* g) {
     fft64_destroy(g);
   cudaFree(g->Q);
   cudaFree(g->E);
+  cudaFree(g->dE);
   cudaFree(g->host_stage);
   copy_streams_destroy(g->copies);
   cudaFree(g->n_out);

@@ -128,6 +128,7 @@ void bunch_kick(const sc_batch* B, int b, KPParams& P, double kl) {
   set_kick(P, g, kl, 1.0);  // batch grids are not sliced: no longitudinal kick
   const size_t off = (size_t)B->idx[b] * cells_of(g);
   P.E = g->E + off;
+  P.dE = g->dE ? g->dE + off : nullptr;
   P.E32 = (const float2*)g->E + off;
 }
 

@@ -210,15 +210,13 @@ SC_HD int fix_split(const FixAxis& a, double x, int& i, int& w, uint64_t& z) {
   return (uint32_t)i < (uint32_t)a.limit ? 1 : 0;
 }
 
-// The fraction xi - i of a decided coordinate, as a double (to 2^-52): its
-// bits under the exponent of 1, less 1 (one FP64 instruction).
+// The fraction xi - i of a decided coordinate, as a double (its leading bits
+// truncated at 2^-F), by shifting its leading bit into place.
 SC_HD double fix_fraction(const FixAxis& a, uint64_t z) {
-  const uint64_t fr = ((z - a.t) << (64 - a.f)) >> 12;
-#if defined(__CUDA_ARCH__)
-  return __dsub_rn(bits_f64(0x3ff0000000000000ull | fr), 1.0);
-#else
-  return bits_f64(0x3ff0000000000000ull | fr) - 1.0;
-#endif
+  const uint64_t fr = (z - a.t) << (64 - a.f);  // in units of 2^-64
+  if (fr == 0) return 0.0;
+  const int n = clz64(fr);
+  return bits_f64(((uint64_t)(1021 - n) << 52) + ((fr << n) >> 11));  // the leading bit adds one to the exponent
 }
 
 }  // namespace sc

@@ -96,6 +96,7 @@ struct KPParams {
   // gather + kick
   GridGeom gk;
   const double2* E;  // (Ex, Ey) per node of the kick grid
+  const double2* dE; // their differences to the next node along x (float64 fields)
   double kl;         // K * L_sc
   int do_kick;
   // Cell cache: the deposit of the previous step located every particle on
@@ -229,6 +230,7 @@ struct sc_grid {
   int device;
   unsigned long long* Q;      // [nstack][ny][nx] uint64 charge (2^40 per particle)
   double2* E;                 // [nstack][ny][nx] (Ex, Ey); float32 pairs in the first half when field32
+  double2* dE;                // [nstack][ny][nx] E(i+1) - E(i) along x, 0 at the last node (float64 fields only)
   int field32;                // the solve writes float32 fields (SC_SOLVE_TF32X3)
   unsigned long long* n_out;  // device counter (one per stacked grid in a batch class)
   unsigned long long* n_nan;  // device counter of non-finite particles seen by deposits (n_out + nstack)

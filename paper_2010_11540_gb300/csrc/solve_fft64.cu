@@ -98,12 +98,14 @@ __global__ void fft64_columns(const double2* __restrict__ F1, int nx, int ny, co
 
 // blockDim.x = nx; block (row, stacked grid)
 __global__ void fft64_rows_inv(const double2* __restrict__ Hx, const double2* __restrict__ Hy, int nx,
-                               double inv_norm, double2* __restrict__ E, const double2* __restrict__ twx) {
+                               double inv_norm, double2* __restrict__ E, double2* __restrict__ dE,
+                               const double2* __restrict__ twx) {
   extern __shared__ double2 sm[];
   const int Mx = 2 * nx, j = blockIdx.x, t = threadIdx.x;
   double2 *A = sm, *B = sm + Mx;
   const size_t so = (size_t)blockIdx.y * gridDim.x * (nx + 1);  // slice blockIdx.y
-  E += (size_t)blockIdx.y * gridDim.x * nx;
+  E += ((size_t)blockIdx.y * gridDim.x + j) * nx;
+  dE += ((size_t)blockIdx.y * gridDim.x + j) * nx;
   const double2* hx = Hx + so + (size_t)j * (nx + 1);
   const double2* hy = Hy + so + (size_t)j * (nx + 1);
   pdl_wait();
@@ -117,7 +119,11 @@ __global__ void fft64_rows_inv(const double2* __restrict__ Hx, const double2* __
   __syncthreads();
   const double2* r = fft_stages<true, true>(A, B, Mx, 2, t, twx);
   pdl_allow();
-  E[(size_t)j * nx + t] = make_double2(r[t].x * inv_norm, r[t].y * inv_norm);
+  const double2 e = make_double2(__dmul_rn(r[t].x, inv_norm), __dmul_rn(r[t].y, inv_norm));
+  E[t] = e;
+  // (r holds nx values; the last node has no next one)
+  const double2 f = r[t + 1 < nx ? t + 1 : t];
+  dE[t] = make_double2(__dsub_rn(__dmul_rn(f.x, inv_norm), e.x), __dsub_rn(__dmul_rn(f.y, inv_norm), e.y));
 }
 
 // Iterative radix-2 FFT on the host (used once per grid for the kernel spectra).
@@ -247,7 +253,8 @@ sc_status fft64_solve(sc_grid* g, bool zero_q) {
                      (const double2*)f.F1, nx, ny, (const double*)f.Sx, (const double*)f.Sy, f.Hx, f.Hy,
                      (const double2*)f.twy, zero_q ? g->Q : (unsigned long long*)nullptr));
   SC_CUDA(launch_pdl(fft64_rows_inv, dim3(ny, nz), dim3(nx), 2 * Mx * sizeof(double2), g->stream, (const double2*)f.Hx,
-                     (const double2*)f.Hy, nx, 1.0 / ((double)Mx * (double)My), g->E, (const double2*)f.twx));
+                     (const double2*)f.Hy, nx, 1.0 / ((double)Mx * (double)My), g->E, g->dE,
+                     (const double2*)f.twx));
   return SC_OK;
 }
 

@@ -102,7 +102,7 @@ __global__ void pipe_rows_inv(const double* __restrict__ T2, int nx, int ny, dou
 
 // One thread per node of every stacked grid.
 __global__ void pipe_fields(const double* __restrict__ phi, int nx, int ny, int nstack, double inv2hx,
-                            double inv2hy, double2* __restrict__ E) {
+                            double inv2hy, double2* __restrict__ E, double2* __restrict__ dE) {
   pdl_wait();
   const int64_t total = (int64_t)nstack * nx * ny;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (int64_t)gridDim.x * blockDim.x) {
@@ -110,11 +110,16 @@ __global__ void pipe_fields(const double* __restrict__ phi, int nx, int ny, int 
     const double* p = phi + (c - (int64_t)j * nx - i);  // this grid's row 0
     const double* row = p + (size_t)j * nx;
     // odd extension across the walls: phi(-1) = -phi(1), phi(n) = -phi(n-2)
-    const double xr = (i + 1 < nx) ? row[i + 1] : -row[nx - 2];
-    const double xl = (i > 0) ? row[i - 1] : -row[1];
-    const double yu = (j + 1 < ny) ? p[(size_t)(j + 1) * nx + i] : -p[(size_t)(ny - 2) * nx + i];
-    const double yd = (j > 0) ? p[(size_t)(j - 1) * nx + i] : -p[(size_t)nx + i];
-    E[c] = make_double2(-(xr - xl) * inv2hx, -(yu - yd) * inv2hy);
+    auto field = [&](int i) {
+      const double xr = (i + 1 < nx) ? row[i + 1] : -row[nx - 2];
+      const double xl = (i > 0) ? row[i - 1] : -row[1];
+      const double yu = (j + 1 < ny) ? p[(size_t)(j + 1) * nx + i] : -p[(size_t)(ny - 2) * nx + i];
+      const double yd = (j > 0) ? p[(size_t)(j - 1) * nx + i] : -p[(size_t)nx + i];
+      return make_double2(__dmul_rn(-(xr - xl), inv2hx), __dmul_rn(-(yu - yd), inv2hy));
+    };
+    const double2 e = field(i), f = i + 1 < nx ? field(i + 1) : e;
+    E[c] = e;
+    dE[c] = make_double2(__dsub_rn(f.x, e.x), __dsub_rn(f.y, e.y));
   }
 }
 
@@ -189,7 +194,7 @@ sc_status pipe_solve(sc_grid* g, bool zero_q) {
   const int64_t total = (int64_t)nz * nx * ny;
   const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 8);
   SC_CUDA(launch_pdl(pipe_fields, dim3(blocks), dim3(256), 0, g->stream, (const double*)f.phi, nx, ny, (int)nz,
-                     0.5 / g->hx, 0.5 / g->hy, g->E));
+                     0.5 / g->hx, 0.5 / g->hy, g->E, g->dE));
   return SC_OK;
 }
 
