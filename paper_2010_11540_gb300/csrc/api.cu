@@ -437,6 +437,10 @@ sc_status create_grid(sc_grid** out, int nx, int ny, double xmin, double xmax, d
   g->geom.ay = make_fix_axis(ymin, g->geom.inv_hy, ny - 1);
   if (n_slices > 1) g->geom.az = make_fix_axis(zmin, g->geom.inv_dz, n_slices);
   g->geom.fix = g->geom.ax.top && g->geom.ay.top && (n_slices == 1 || g->geom.az.top);
+  g->sum_axes.x = make_sum_axis(xmin, g->geom.inv_hx, nx - 1);
+  g->sum_axes.y = make_sum_axis(ymin, g->geom.inv_hy, ny - 1);
+  if (n_slices > 1) g->sum_axes.z = make_sum_axis(zmin, g->geom.inv_dz, n_slices);
+  g->sum_axes.usable = g->sum_axes.x.f && g->sum_axes.y.f && (n_slices == 1 || g->sum_axes.z.f);
   tile_window(nx, ny, &g->geom.wx0, &g->geom.wy0, &g->geom.wnx, &g->geom.wny);
   sc_status st = SC_OK;
   cudaError_t e = cudaGetDevice(&g->device);

@@ -122,6 +122,10 @@ __device__ __forceinline__ void add4(unsigned long long* Q, int nx, int cell, co
   atomicAdd(q + nx, w[2]);
   atomicAdd(q + nx + 1, w[3]);
 }
+// (A tile's high word is 0 for one weight in forty: skipping its add pays in
+// the kick/push, 0.7% of a turn, and costs 3% in the stand-alone deposit, whose
+// integer slots are the scarce ones: ALWAYS.)
+template <bool ALWAYS = false>
 __device__ __forceinline__ void add4(const Tile& t, int nx, int cell, const unsigned long long (&w)[4]) {
   const int c[4] = {cell, cell + 1, cell + nx, cell + nx + 1};
   uint32_t old[4];
@@ -131,7 +135,7 @@ __device__ __forceinline__ void add4(const Tile& t, int nx, int cell, const unsi
   for (int k = 0; k < 4; ++k) {
     const uint32_t l = (uint32_t)w[k];
     const uint32_t h = (uint32_t)(w[k] >> 32) + (old[k] + l < l ? 1u : 0u);
-    if (h) atomicAdd(t.hi + c[k], h);
+    if (ALWAYS || h) atomicAdd(t.hi + c[k], h);
   }
 }
 template <class Dst>

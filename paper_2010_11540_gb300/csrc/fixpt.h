@@ -219,4 +219,68 @@ SC_HD double fix_fraction(const FixAxis& a, uint64_t z) {
   return bits_f64(((uint64_t)(1021 - n) << 52) + ((fr << n) >> 11));  // the leading bit adds one to the exponent
 }
 
+// The leading 64 bits of a b from three 32 x 32-bit products, short by at most three units.
+SC_HD uint64_t mulhi64_near(uint64_t a, uint64_t b) {
+  const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+#if defined(__CUDA_ARCH__)
+  const uint32_t m1 = __umulhi(ah, bl), m2 = __umulhi(al, bh);
+#else
+  const uint32_t m1 = (uint32_t)(((uint64_t)ah * bl) >> 32), m2 = (uint32_t)(((uint64_t)al * bh) >> 32);
+#endif
+  return (uint64_t)ah * bh + m1 + m2;
+}
+
+// The same decision for kernels that have FP64 slots to spare and integer ones
+// not: the integer of x is read from the bits of x + magic, magic = 1.5 2^k
+// large enough that the sum's last bit is worth the same 2^-s for every x of
+// the grid -- one FP64 instruction in place of some fourteen integer ones.
+// 52 bits instead of 63: F is near 44, one coordinate in 2^18 is undecided.
+struct SumAxis {
+  double magic;
+  uint64_t c;       // inv_h's significand, normalised to 2^63..2^64
+  uint64_t neg_x0;  // minus (the bits of xmin + magic, less what T units of xi are)
+  int32_t f;        // F; 0: not usable
+  uint32_t near;    // 2 T in units of 2^-53 (rounded up)
+  int32_t limit;    // cells
+};
+
+// T: the two roundings' cells 2^-52, one unit each for the sums of x and xmin,
+// three for the product, two for T's own place.
+inline SumAxis make_sum_axis(double xmin, double inv_h, int cells) {
+  SumAxis a{};
+  a.limit = cells;
+  if (!(inv_h > 0.0) || cells < 1 || cells > 4096) return a;
+  const double xmax = xmin + cells / inv_h;
+  const double lo = xmin < 0 ? -xmin : xmin, hi = xmax < 0 ? -xmax : xmax, big = lo > hi ? lo : hi;
+  const int top = (int)(f64_bits(big) >> 52), ei = (int)(f64_bits(inv_h) >> 52);
+  if (top < 100 || top > 1946 || ei < 100 || ei > 1946) return a;
+  // |x| < 2^(top - 1022) in the grid: 1.5 2^k + x stays between 2^k and 2^(k+1) for k = top - 1021, its
+  // last bit worth 2^(k - 52)
+  const int s = 1073 - top, f = s + 1022 - ei;
+  if (f < 34 || f > 62) return a;
+  const uint64_t t = (uint64_t)((((unsigned __int128)(cells + 1) << f) >> 52) + 1) + 8;
+  if ((2 * t) >> (f - 28)) return a;  // 2 T above 2^-7 of the spacing of the places: too many undecided
+  a.magic = bits_f64((uint64_t)(top + 2) << 52 | 1ull << 51);
+  a.c = ((f64_bits(inv_h) & ((1ull << 52) - 1)) | (1ull << 52)) << 11;
+  a.neg_x0 = (uint64_t)((((unsigned __int128)t) << 64) / a.c) + 1 - f64_bits(xmin + a.magic);
+  a.near = (uint32_t)(((unsigned __int128)(2 * t) << (85 - f)) >> 32) + 1;
+  a.f = f;
+  return a;
+}
+
+// As fix_split.  (Coordinates below the grid, infinities and NaN wrap to
+// integers beyond its end: the bits of the sum grow with it.)
+SC_HD int sum_split(const SumAxis& a, double x, int& i, int& w) {
+#if defined(__CUDA_ARCH__)
+  const double v = __dadd_rn(x, a.magic);
+#else
+  const double v = x + a.magic;
+#endif
+  const uint64_t z = mulhi64_near(f64_bits(v) + a.neg_x0, a.c);
+  i = (int)((uint32_t)(z >> 32) >> (a.f - 32));
+  w = (int)((((uint32_t)(z >> (a.f - 21)) - ((uint32_t)i << 21)) + 1u) >> 1);
+  if ((uint32_t)((z << (85 - a.f)) >> 32) < a.near) return -1;
+  return (uint32_t)i < (uint32_t)a.limit ? 1 : 0;
+}
+
 }  // namespace sc

@@ -75,6 +75,12 @@ struct GridGeom {
   int fix;
 };
 
+// The axes as the stand-alone deposit decides cells (x, y, and sigma when sliced); usable: all of them.
+struct SumAxes {
+  SumAxis x, y, z;
+  int usable;
+};
+
 // Shared memory of a block's deposit tile (uint64 per node of its window).
 constexpr int kTileBytes = 200 * 1024;
 
@@ -225,6 +231,7 @@ struct sc_grid {
   double zmin, zmax;
   double xmin, xmax, ymin, ymax, hx, hy;
   sc::GridGeom geom;
+  sc::SumAxes sum_axes;        // for the stand-alone deposit
   cudaStream_t stream;
   bool own_stream;
   int device;

@@ -23,6 +23,8 @@ HARNESS = r"""
 #include "fixpt.h"
 using namespace sc;
 static long bad = 0, unsure = 0, seen = 0;
+static bool sum;
+static SumAxis sx;
 static void one(const FixAxis& ax, double x, double xmin, double inv, int cells) {
   const volatile double d = x - xmin;
   const volatile double xi = d * inv;
@@ -30,12 +32,12 @@ static void one(const FixAxis& ax, double x, double xmin, double inv, int cells)
   double f = 0;
   const bool in = cic_split(xi, cells, i, a, &f);
   int gi, gw;
-  uint64_t z;
-  const int r = fix_split(ax, x, gi, gw, z);
+  uint64_t z = 0;
+  const int r = sum ? sum_split(sx, x, gi, gw) : fix_split(ax, x, gi, gw, z);
   ++seen;
   if (r < 0) { ++unsure; return; }
   bool ok = (r == 1) == in;
-  if (ok && in) ok = gi == i && gw == a && fabs(fix_fraction(ax, z) - f) <= (cells + 1) * 0x1p-52 + 0x1p-52;
+  if (ok && in) ok = gi == i && gw == a && (sum || fabs(fix_fraction(ax, z) - f) <= (cells + 1) * 0x1p-52 + 0x1p-52);
   if (!ok && ++bad < 6) printf("bad x %.17g xi %.17g in %d/%d i %d/%d w %d/%d\n", x, xi, r, in, gi, i, gw, a);
 }
 int main(int argc, char** argv) {
@@ -43,7 +45,9 @@ int main(int argc, char** argv) {
   const int n = atoi(argv[3]), cells = n - 1;
   const double h = (xmax - xmin) / cells, inv = 1.0 / h;
   const FixAxis ax = make_fix_axis(xmin, inv, cells);
-  if (!ax.top) { printf("off\n"); return 0; }
+  sum = argc > 4 && argv[4][0] == 's';
+  sx = make_sum_axis(xmin, inv, cells);
+  if (sum ? !sx.f : !ax.top) { printf("off\n"); return 0; }
   std::mt19937_64 g(n);
   std::uniform_real_distribution<double> U(0, 1);
   for (long k = 0; k < 2000000; ++k) one(ax, xmin + (xmax - xmin) * (1.2 * U(g) - 0.1), xmin, inv, cells);
@@ -80,15 +84,24 @@ def harness(tmp_path_factory):
     return d / "h"
 
 
+@pytest.mark.parametrize("kind", ["bits", "sum"])
 @pytest.mark.parametrize("xmin,xmax,n", [
     (-0.02, 0.02, 128), (-0.015, 0.015, 256), (-0.01, 0.01, 64), (-0.02, 0.02, 129), (0.0, 1.0, 16), (-0.012, 0.009, 33),
     (0.01, 0.02, 512), (-0.03, -0.01, 65), (-60.0, 60.0, 33), (-1e-9, 1e-9, 128), (-4.0, 4.0, 4097), (-1e6, 1e6, 9),
     (-0.02, 1e-7, 100), (1000.0, 1000.5, 64), (-0.02, 0.02, 2)])
-def test_decides_as_the_two_roundings(harness, xmin, xmax, n):
-    out = subprocess.run([str(harness), repr(xmin), repr(xmax), str(n)], check=True, capture_output=True, text=True).stdout
+def test_decides_as_the_two_roundings(harness, xmin, xmax, n, kind):
+    out = subprocess.run([str(harness), repr(xmin), repr(xmax), str(n), kind], check=True, capture_output=True,
+                         text=True).stdout
+    if kind == "sum" and out.strip() == "off":  # too few bits for this axis: the caller keeps cic_split
+        assert xmin >= 1000.0
+        return
     bad, unsure, seen = map(int, out.split()[-3:])
     assert bad == 0, out
-    assert unsure <= 20 + seen * 2.0 ** -7 * (1 if xmin >= 100 else 2.0 ** -8), out
+    if kind == "bits":
+        share = 2.0 ** -7 * (1 if xmin >= 100 else 2.0 ** -8)
+    else:  # 2 T of each 2^(F - 21) units, T <= 10, F >= 50 - log2(cells) (less what an off-centre grid loses)
+        share = 20 * (n - 1) * 2.0 ** -29 * max(1.0, 2 * max(abs(xmin), abs(xmax)) / (xmax - xmin))
+    assert unsure <= 20 + seen * share, out
 
 
 def test_unusable_axes_are_refused(harness):
