@@ -6,6 +6,7 @@
 // flushed once per block.  One thread per
 // particle, persistent grid over SoA float64 state; one launch serves one grid
 // (kick_push_kernel) or every bunch of a batch (kick_push_batched).
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -417,9 +418,15 @@ int kick_push_blocks_at(int smem_bytes, bool tile, bool f32, int threads) {
 // 25.5 -> 22.6 us, 128^2 28.1 -> 27.6, 256^2 68.5 -> 66.9; 5e4: 64^2 25.6 ->
 // 23.2, but 256^2 68.8 -> 86.4; 1e5: 64^2 26.1 -> 26.3).
 int default_threads(int64_t n, bool f32, int smem) {
+  // the device's SM count, asked for once per device ordinal (a query per launch showed in small calls)
+  static std::atomic<int> known[64];
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (dev >= 0 && dev < 64) sms = known[dev].load(std::memory_order_relaxed);
+  if (sms == 0) {
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (dev >= 0 && dev < 64) known[dev].store(sms, std::memory_order_relaxed);
+  }
   return n <= (int64_t)sms * (smem <= 32 * 1024 ? 384 : 192) ? 384 : kick_push_max_threads(f32);
 }
 

@@ -189,15 +189,17 @@ def create_grid(nx, ny, xmin, xmax, ymin, ymax, precision="fp64", stream=None, s
 
 def particles(state) -> Particles:
     """sc_particles from a dict of six CUDA float64 contiguous tensors of equal length."""
-    keys = ("x", "px", "y", "py", "sigma", "psigma")
-    ts = [state[k] for k in keys]
-    n = int(ts[0].numel())
+    # (a small call's time is mostly this: each tensor attribute costs some 60 ns, so the dtype is
+    # looked at once and compared)
+    x, px, y, py, sg, ps = ts = (state["x"], state["px"], state["y"], state["py"], state["sigma"], state["psigma"])
+    n, dtype = x.numel(), x.dtype
+    float64 = dtype.is_floating_point and x.element_size() == 8
     for t in ts:
-        if not (t.is_cuda and t.dtype.is_floating_point and t.element_size() == 8 and t.is_contiguous()):
+        if not (float64 and t.is_cuda and t.dtype is dtype and t.is_contiguous()):
             raise ValueError("particle arrays must be contiguous CUDA float64 tensors")
         if t.numel() != n:
             raise ValueError("particle arrays differ in length")
-    return Particles(*(t.data_ptr() for t in ts), n)
+    return Particles(x.data_ptr(), px.data_ptr(), y.data_ptr(), py.data_ptr(), sg.data_ptr(), ps.data_ptr(), n)
 
 
 def beam(b: dict) -> Beam:
