@@ -582,6 +582,9 @@ sc_status sc_kick_push(sc_grid* g, const sc_particles* p, const sc_beam* b, doub
   KPParams P = base_params(p, b);
   set_kick(P, g, kick_strength(b) * L_sc, b->gamma0);
   if (next) set_deposit(P, next);
+  // the gather reads g's fields, whatever `next` solves with (without a cell cache the deposit has no field type)
+  P.field32 = g->field32;
+  P.series = series_drift(g);
   if (n_elems > KP_INLINE) {
     // long segment: compiled copy in device memory (synchronous upload)
     std::vector<DevElem> dev(n_elems);
