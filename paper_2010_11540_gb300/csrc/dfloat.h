@@ -121,6 +121,22 @@ SC_HD F2 rsqrt1m_series(F2 u) {
   return F2{wh, f_add(f_fma(0.5f, u.l, f_add(f_sub(uh, wh), z.h)), z.l)};
 }
 
+// (1 - u)^(-1/2) - 1 over the wider range |u| < 2^-7 (either sign),
+//   u/2 + u^2 (3/8 + u (5/16 + u (35/128 + 63/256 u + 231/1024 u^2 + 429/2048 u^3))),
+// absolute error below 2^-53: the leading sum's own 2^-46 of 2^-8, halved by its
+// rounding; the innermost float part's u 2^-25 enters times u^4, and the next
+// term is 6435/32768 u^8 < 2^-58.
+constexpr float kSlopeMaxU = 0.0078125f;
+SC_HD F2 rsqrt1m_wide(F2 u) {
+  const float s = f_mul(u.h, f_fma(u.h, f_fma(u.h, 0.20947265625f, 0.2255859375f), 0.24609375f));
+  const float qh = f_add(0.2734375f, s);
+  const F2 q{qh, f_add(f_sub(0.2734375f, qh), s)};
+  const F2 t = f2_add(F2{0.3125f, 0.f}, f2_mul(u, q));
+  const F2 v = f2_add(F2{0.375f, 0.f}, f2_mul(u, t));
+  const F2 z = f2_mul(f2_sqr(u), v);
+  return f2_add(F2{f_mul(0.5f, u.h), f_mul(0.5f, u.l)}, z);
+}
+
 // 1 - sqrt(1 - v) for |v| < 2^-9 by its power series,
 //   v/2 + v^2 (1/8 + v/16 + 5/128 v^2 + 7/256 v^3 + 21/1024 v^4),
 // absolute error below 2^-54 (next term 33/2048 v^7 < 2^-68; the bracket's

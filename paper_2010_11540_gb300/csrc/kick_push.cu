@@ -214,14 +214,14 @@ __device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile
       }
     }
     if (!F32 && kept) load_psc();
-    if (!kept) ps_const<SERIES>(k, s.ps, P.beta0_sq, fresh || P.has_quad != 0);
+    if (!kept) ps_const<SERIES, F32, CACHE>(k, s.ps, P.beta0_sq, fresh || P.has_quad != 0);
     const bool quads = psc_mode != 0 || P.has_quad != 0;
     // the quadrupole coefficient cache holds this particle's values unless ps changed in this launch
     const double* qc = (P.qcache && psc_mode == 1 && !fresh) ? P.qcache + p : nullptr;
     const double* psp = (P.ps_mode & 2) ? P.ps + p : nullptr;
     const bool changed =
-        P.el ? push_elements<XE, SERIES>(s, k, P.el, P.n_elem, P.beta0_sq, P.inv_gamma0_sq, quads, qc, n, psp)
-             : push_elements<XE, SERIES>(s, k, P.inl, P.n_elem, P.beta0_sq, P.inv_gamma0_sq, quads, qc, n, psp);
+        P.el ? push_elements<XE, SERIES, F32>(s, k, P.el, P.n_elem, P.beta0_sq, P.inv_gamma0_sq, quads, qc, n, psp)
+             : push_elements<XE, SERIES, F32>(s, k, P.inl, P.n_elem, P.beta0_sq, P.inv_gamma0_sq, quads, qc, n, psp);
     if (fresh || (psc_mode == 1 && changed)) {
       P.psc[p] = k.d0;
       P.psc[n + p] = k.d1;

@@ -77,11 +77,48 @@ __device__ __forceinline__ F2 slip(double d, double r0) {
   return slip_general(d, r0);
 }
 
-template <bool SERIES>
+// r0 = 1/(1+delta) as y (1 + eps).  Where v = (1+delta)^2 - 1 = 2 ps + beta0^2
+// ps^2 lies within 2^-7 of 0 (|ps| below 3.9e-3), r0 = 1 + ((1 + v)^(-1/2) - 1)
+// with the bracket in float pairs (v to 2^-46 of itself: r0 to 2^-55) takes two
+// FP64 instructions where the refined reciprocal root and its residual take
+// fourteen (WIDE; float32 fields).  A stand-alone kick/push computes it for
+// every particle: one cell of 4e6 particles on 256^2, split TF32, 1621 -> 1418
+// us.  With a plan it is computed once per call and after RF cavities, and is
+// called there (CALL): inlined, its code made a turn 1% slower that never ran
+// it (called: 14.95 -> 14.88 ms).  Float64 fields keep the root: there either
+// form spills more in the turn's kernel (18.0 -> 18.3 ms), and the two paths are
+// to round alike.
+struct InvDelta {
+  double y;
+  float eps;
+};
+__device__ __forceinline__ InvDelta inv_delta(double ps, double beta0_sq) {
+  const F2 p = f2_split(ps);
+  const F2 v = f2_add(f2_mul(f2_sqr(p), f2_split(beta0_sq)), F2{2.f * p.h, 2.f * p.l});
+  InvDelta r;
+  if (abs_hi(ps) < 0x3fe00000u && fabsf(v.h) < kSlopeMaxU) {
+    const F2 c = rsqrt1m_wide(f2_neg(v));
+    r.y = 1.0 + f2_to_double(c);
+    const F2 rest = f2_add(c, f2_neg(f2_split(r.y - 1.0)));  // (relative to r0, which is 1 to 2^-8)
+    r.eps = f_add(rest.h, rest.l);
+  } else {
+    r.y = rsqrt_split(opd_sq(ps, beta0_sq), r.eps);
+  }
+  return r;
+}
+__device__ __noinline__ InvDelta inv_delta_call(double ps, double beta0_sq) { return inv_delta(ps, beta0_sq); }
+
+template <bool SERIES, bool WIDE, bool CALL>
 __device__ __forceinline__ void ps_const(PsConst& k, double ps, double beta0_sq, bool quads) {
   k.eps = 0.f;
   if (SERIES) {
-    k.d0 = rsqrt_split(opd_sq(ps, beta0_sq), k.eps);
+    if (WIDE) {
+      const InvDelta r0 = CALL ? inv_delta_call(ps, beta0_sq) : inv_delta(ps, beta0_sq);
+      k.d0 = r0.y;
+      k.eps = r0.eps;
+    } else {
+      k.d0 = rsqrt_split(opd_sq(ps, beta0_sq), k.eps);
+    }
     k.d1 = f2_pack(slip((1.0 - beta0_sq) * ps * fma(beta0_sq, ps, 2.0), k.d0));
   } else {
     k.d0 = opd_sq(ps, beta0_sq);
@@ -381,8 +418,9 @@ __device__ __forceinline__ void map_rf(State& s, const DevElem& e) {
 // the state does not hold it (segments of drifts and thin sextupoles), else
 // NULL.  XE: the segment may hold thick sextupoles or exact dipoles (their
 // code is compiled only into the kernels that need it, keeping the common
-// kernels' registers).  SERIES: which drift (and which d0, d1 of k).
-template <bool XE, bool SERIES>
+// kernels' registers).  SERIES: which drift (and which d0, d1 of k); WIDE: see
+// ps_const.
+template <bool XE, bool SERIES, bool WIDE>
 __device__ __forceinline__ bool push_elements(State& s, PsConst& k, const DevElem* __restrict__ el, int n_elem,
                                               double beta0_sq, double inv_gamma0_sq, bool quads,
                                               const double* __restrict__ qc, size_t n, const double* psp) {
@@ -423,7 +461,7 @@ __device__ __forceinline__ bool push_elements(State& s, PsConst& k, const DevEle
         c.sg = F2{0.f, 0.f};
         c.has_sg = c.has_rr = false;
         map_rf(s, e);
-        ps_const<SERIES>(k, s.ps, beta0_sq, quads);
+        ps_const<SERIES, WIDE, true>(k, s.ps, beta0_sq, quads);
         changed = true;
         break;
       default: break;

@@ -61,6 +61,14 @@ int main() {
       see(val(one_minus_sqrt1m(v)) - x / (1 + sqrtl(1 - x)), p53);
     }
   printf("sqrt %.3f\n", worst); worst = 0;
+  for (int e = -60; e <= -7; ++e)
+    for (int i = 0; i < 4000; ++i) {
+      const double sgn = U(g) < 0 ? -1 : 1;
+      const F2 u = f2_split(sgn * ldexp(1.0 - 0.5 * fabs(U(g)) - 1e-9, e));
+      const Q x = val(u);
+      see(val(rsqrt1m_wide(u)) - x / (sqrtl(1 - x) * (1 + sqrtl(1 - x))), ldexpl(1, -53));
+    }
+  printf("wide %.3f\n", worst); worst = 0;
   for (int i = 0; i < 200000; ++i) {
     double d[12];
     for (double& v : d) v = U(g) * ldexp(1.0, (int)(U(g) * 12));
@@ -97,6 +105,6 @@ def results(tmp_path_factory):
     return {k: float(v) for k, v in (line.split() for line in out.splitlines())}
 
 
-@pytest.mark.parametrize("what", ["split", "edges", "rsqrt", "sqrt", "slip"])
+@pytest.mark.parametrize("what", ["split", "edges", "rsqrt", "sqrt", "wide", "slip"])
 def test_within_the_stated_bound(results, what):
     assert results[what] <= 1.0, results

@@ -70,3 +70,23 @@ def test_not_finite_and_huge(precision):
         fin = np.isfinite(ref[k])
         assert np.array_equal(fin, np.isfinite(got[k])), k
         assert np.allclose(got[k][fin], ref[k][fin], rtol=1e-13, atol=1e-13), k
+
+
+@pytest.mark.parametrize("ps", [0.0, 2e-16, 1e-3, 0.0039, 0.00392, -0.0039, -0.00392, 0.05])
+def test_inverse_delta_on_both_sides_of_its_series(ps):
+    """1/(1+delta) as a series and, from |2 ps + beta0^2 ps^2| = 2^-7 on, as a root: a long drift of small slopes."""
+    n, L, b = 257, 1000.0, synth.beam()
+    rng = np.random.default_rng(5)
+    parts = {k: rng.uniform(-1.0, 1.0, n) * s for k, s in
+             zip(KEYS, (8e-3, 2e-3, 8e-3, 2e-3, 10.0, 0.0))}
+    parts["psigma"] = ps * (1.0 + 1e-3 * rng.uniform(-1.0, 1.0, n))
+    table = synth.table([synth.elem(synth.DRIFT, L)])
+    st = to_gpu(parts)
+    sc.kick_push(sc.create_grid(64, 64, -0.02, 0.02, -0.015, 0.015, precision="tf32x3"), st, b, 0.0, table)
+    got, ref = to_host(st), oracle.copy_state(parts)
+    oracle.push(ref, table, b)
+    for k in KEYS:  # bounds as above
+        size = np.abs(ref[k]) + np.abs(parts[k]) + L * (np.abs(parts["px"]) + np.abs(parts["py"])) + 1e-12
+        if k == "sigma":
+            size = size + L
+        assert np.all(np.abs(got[k] - ref[k]) <= 32 * 2.0 ** -52 * size), k
