@@ -54,7 +54,7 @@ FP64_INST = {"base": 17.5, "drift": 12.2, "quad": 20.6, "sext": 5.0, "bend": 16.
 FP64_INST_QUAD_UNCACHED = 51.0  # with the longitudinal kick (psigma changes at every kick: no cache); earlier build
 # split-TF32 form: float32 gather from the cached fixed-point weights
 FP64_INST_BASE_F32 = 5.8
-# sliced grids: the slice index (one subtract, one multiply; the floor is integer work) per locate
+# sliced grids: the slice index (one subtract, one multiply) per locate, in the all-FP64 work
 FP64_INST_SLICE = 2.0
 # Bezier gather instead of bilinear fields (extra per particle-kick), and the
 # longitudinal kick (bilinear / Bezier potentials of two slices plus the
@@ -70,17 +70,15 @@ FP64_INST_LON_BEZIER_F32 = 13.95
 # cache; c2: mean of the three segment types), with the kernel sources'
 # SHA-256 (first 16 hex digits) they were captured on: the roofline's
 # "traffic" while the sources still match; other workloads report null.
-KP_TRAFFIC_TF32 = {"c2": (127.4e6, "07458f3c69a23e63"),  # 1e6 particles (the working set partly stays in L2)
+KP_TRAFFIC_TF32 = {"c2": (127.4e6, "d99a731ba8300420"),  # 1e6 particles (the working set partly stays in L2)
                    "c4": (3860.0e6, "052c41cbfc714941"),  # 2.37e7 particles, batched (kick_push_traffic_c4_c5.md)
                    "c5": (1594.1e6, "052c41cbfc714941")}  # 1e7 particles in 32 slices
 # GB300: 152 SMs x 2 FP64 instructions per SM clock x 2.07 GHz maximum clock
 FP64_PIPE_PEAK_TINST = 152 * 2 * 2.07e9 / 1e12
-# FP64-pipe instructions per particle of the stand-alone deposit (xi and eta: a
-# subtract and a multiply each, 4.23 measured with ncu
-# sm__thread_inst_executed_pipe_fp64_pred_on, profiles/deposit_c2.md; the
-# slice index two more)
-DEP_FP64_INST = 4.23
-DEP_FP64_INST_SLICE = 2.0
+# FP64-pipe instructions per particle of the stand-alone deposit: one sum per
+# axis (csrc/fixpt.h, sum_split), the slice one more
+DEP_FP64_INST = 2.0
+DEP_FP64_INST_SLICE = 1.0
 # What the kernels of the tree issue to the FP64 pipe, measured the same way on
 # the sources whose SHA-256 (first 16 hex digits) is FP64_INST_SOURCES_SHA:
 # corrections and the path length in float pairs (csrc/dfloat.h).  By kernel
@@ -92,7 +90,7 @@ FP64_ISSUED = {
     "f32": {"base": 2.76, "drift": 11.2, "quad": 8.61, "sext": 5, "bend": 16.0, "rf": 30.0},
 }
 KP_SOURCES = ("kick_push.cu", "maps.cuh", "cic.cuh", "fixpt.h", "dfloat.h", "sc_internal.cuh")
-FP64_INST_SOURCES_SHA = "07458f3c69a23e63"
+FP64_INST_SOURCES_SHA = "d99a731ba8300420"
 # HBM bytes per particle-kick that the fused kick/push must move (algorithmic):
 # the six float64 coordinates read (48 B) and the five a kick and a push
 # change written back (40 B: psigma changes only in RF cavities); 96 B when
@@ -217,7 +215,7 @@ def fp64_issued_per_kick(lat, precision, sliced):
     """FP64-pipe instructions per particle-kick that the kernels of the tree issue."""
     fam = "f64" if precision in ("fp64", "pipe_fp64") else "f32_series" if precision == "tf32x3" and not sliced else "f32"
     t, mix = FP64_ISSUED[fam], element_mix(lat)
-    f = mix["kicks"] * (t["base"] + (FP64_INST_SLICE if sliced else 0.0))
+    f = mix["kicks"] * t["base"]  # (sliced grids find the slice in integers)
     return (f + sum(mix[k] * t[k] for k in ("drift", "quad", "sext", "bend", "rf"))) / mix["kicks"]
 
 
@@ -508,7 +506,7 @@ class SingleRun:
                                "consecutive words, measured in this run",
                 "context_peak_random_words": atom_random / 1e9,
                 "frac_of_random_words": rate / atom_random, "ordered_bunch": ordered,
-                # what binds it: the locate's FP64 subtract and multiply per axis (the cell, fraction and
+                # what binds it: the locate's FP64 sum per axis and integer issue (the cell, fraction and
                 # weights are decoded from the bits with integer instructions), on the 2-per-clock FP64 pipe
                 "fp64_pipe": {"fp64_inst_per_particle": DEP_FP64_INST + (DEP_FP64_INST_SLICE if self.slices else 0),
                               "achieved": (DEP_FP64_INST + (DEP_FP64_INST_SLICE if self.slices else 0)) * self.n

@@ -351,8 +351,9 @@ sc_status sc_set_solver_tiling(sc_grid *g, const int *choice);
  * 16 space-charge steps (solve, then kick/push with its deposit), captured as
  * a graph, on a scratch copy of the bunch, and the fastest is kept (the
  * particles, the charge grid and the out-of-grid counter are left as they
- * were); smaller bunches take the largest block and the field type's default
- * traversal.  A re-capture for the same particles, beam, lattice and options
+ * were); smaller bunches take the largest block (launched as 384-thread
+ * blocks when the bunch would fill few SMs with largest ones) and the field
+ * type's default traversal.  A re-capture for the same particles, beam, lattice and options
  * (tracing or diagnostics switched) reuses the choice.
  * sc_set_kick_push_shape fixes either part (the next sc_track_turns
  * re-captures); sc_get_kick_push_shape reads the shape of the captured turn

@@ -36,7 +36,8 @@ __device__ __noinline__ int locate_exact(const GridGeom& g, double x, double y, 
 // took 4 of its instructions per particle, 6 on sliced grids, 64 clocks each):
 // for the one particle in some millions that lies too near a place where the
 // decision changes, and on axes the integers do not serve (GridGeom::fix),
-// locate_exact decides.
+// locate_exact decides.  (Stand-alone deposit of 1e6 particles 11.7 -> 10.1 us,
+// 1e7 in 32 slices 130 -> 107 us; one turn of 4e6 particles, BF16, 71.4 -> 64.5 ms.)
 template <bool FRAC>
 __device__ __forceinline__ int locate(const GridGeom& g, double x, double y, double sg, int2& a, double& fx,
                                       double& fy, int& i, int& j, int& k) {
@@ -94,6 +95,8 @@ __device__ __forceinline__ int locate(const GridGeom& g, double x, double y, dou
 // added to by its low word, whose old value gives the carry, and its high word
 // (the sum is exact whatever the order of the adds).  Words of a plane lie
 // next to each other, so a warp's 32 random bins spread over all 32 banks.
+// Against 64-bit bins: stand-alone deposit of 1e6 particles on 128^2 15.2 ->
+// 11.6 us, a 16-bunch batch's turn 118.5 -> 114.7 ms.
 struct Tile {
   uint32_t* lo;
   uint32_t* hi;

@@ -98,7 +98,16 @@ __device__ __noinline__ void store_quad_cache(const KPParams& P, double ps, doub
 // deposit; F32: float32 fields and gather (the split-precision solve's fields
 // carry float32 accuracy; the fractions are then the deposit's own fixed-point
 // weights), else float64 fields and fractions; SERIES: the drift in float
-// pairs (map_drift, series_drift).  Indices are 32-bit (fewer than 2^24
+// pairs (map_drift, series_drift).
+//
+// Bound by the FP64 pipe, which holds a sub-partition for 64 clocks per warp
+// instruction, and beside it by the latency of its own chain at 24 warps per
+// SM; DRAM traffic is a third of what the time would allow.  So the work is in
+// float pairs and integers wherever those are as exact: with 47 -> 18 FP64
+// instructions per particle and kick, the three kinds of launch of the
+// 216-location ring (1e6 particles, 128^2, TF32: drift-quadrupole-drift-
+// sextupole-drift, drift-quadrupoles-drift, one drift) take 74, 78 and 43 us
+// from a cold cache instead of 116, 136 and 53.  Indices are 32-bit (fewer than 2^24
 // particles): 64-bit ones cost another add per array access, 4% of a batch's turn.
 template <bool CACHE, bool F32, bool XE, bool SERIES>
 __device__ __forceinline__ void kick_push_range(const KPParams& P, bool use_tile, void* tile_smem,
@@ -479,7 +488,7 @@ sc_status launch_kick_push_batched(const KPParams* descs, const int4* blocks, in
 // to 1e-5 on sliced grids, whose slices carry 50 times the line density.  Only
 // the first is below 1e-9, so the others keep the general drift and with it
 // the bits of every position and momentum.  One turn, 1e6 particles on 128^2,
-// TF32: series 16.5 ms, general 21.1 ms (float64 fields: 24.2 ms with the series).
+// TF32: series 14.9 ms, general 19.0 ms (float64 fields: 18.0 ms with the series).
 bool series_drift(const sc_grid* g) { return !g->field32 || (g->precision == SC_SOLVE_TF32X3 && g->nz == 1); }
 
 // Per-element constants in float64 on the host (libm), in the layouts that
