@@ -614,7 +614,8 @@ int ps_mode_mask(const sc_element* host, int n, bool lon) {
   bool reads = lon, writes = lon;
   for (int i = 0; i < n; ++i) {
     const sc_element& e = host[i];
-    if (e.type == SC_QUAD || e.type == SC_BEND || e.type == SC_RF || (e.type == SC_SEXT && e.length > 0.0))
+    if (e.type == SC_QUAD || e.type == SC_BEND || e.type == SC_EXACT_BEND || e.type == SC_RF ||
+        (e.type == SC_SEXT && e.length > 0.0))
       reads = true;
     if (e.type == SC_RF) writes = true;
   }
