@@ -29,6 +29,9 @@ enum : int { QF_ZERO = 0, QF_FOCUS_X = 1, QF_FOCUS_Y = 2, QF_KIND = 3, QF_FAM_SH
 // sin/cos/sinh/cosh are used.
 constexpr double kMaxDelta = 0.00390625;
 
+// A g0 of the plan (PsConst) that stands for none: the drift takes its general form.
+constexpr float kNoSlip = 1e30f;
+
 struct State {
   double x, px, y, py, sg, ps;
 };
@@ -67,13 +70,18 @@ __device__ __forceinline__ double rsqrt_split(double a, float& eps) {
 }
 
 // g0 without cancellation: (1+delta)^2 - (1 + beta0^2 ps)^2 = (1 - beta0^2) ps
-// (2 + beta0^2 ps), so with v = that r0^2, g0 = 1 - sqrt(1 - v).
+// (2 + beta0^2 ps), so with v = that r0^2, g0 = 1 - sqrt(1 - v).  That holds
+// for |ps| < 1/2, where (1+delta)^2 and 1 + beta0^2 ps are positive and r0 is
+// below 2^27.  Other psigma (not finite ones among them, which a float pair
+// cannot hold: f2_split only moves bits) get a g0 that map_drift refuses.
 __device__ __noinline__ F2 slip_general(double d, double r0) {
   return f2_split(d * r0 * r0 / (1.0 + sqrt(1.0 - d * r0 * r0)));
 }
-__device__ __forceinline__ F2 slip(double d, double r0) {
+__device__ __forceinline__ F2 slip(double ps, double beta0_sq, double r0) {
+  if (abs_hi(ps) >= 0x3fe00000u) return F2{kNoSlip, 0.f};
+  const double d = (1.0 - beta0_sq) * ps * fma(beta0_sq, ps, 2.0);
   const F2 v = f2_mul(f2_split(d), f2_sqr(f2_split(r0)));
-  if (abs_hi(d) < kHi2p50 && fabsf(v.h) < kSlipMaxV) return one_minus_sqrt1m(v);
+  if (fabsf(v.h) < kSlipMaxV) return one_minus_sqrt1m(v);
   return slip_general(d, r0);
 }
 
@@ -119,7 +127,7 @@ __device__ __forceinline__ void ps_const(PsConst& k, double ps, double beta0_sq,
     } else {
       k.d0 = rsqrt_split(opd_sq(ps, beta0_sq), k.eps);
     }
-    k.d1 = f2_pack(slip((1.0 - beta0_sq) * ps * fma(beta0_sq, ps, 2.0), k.d0));
+    k.d1 = f2_pack(slip(ps, beta0_sq, k.d0));
   } else {
     k.d0 = opd_sq(ps, beta0_sq);
     k.d1 = fma(beta0_sq, ps, 1.0);
@@ -165,8 +173,8 @@ __device__ __forceinline__ double drift_general(State& s, double L, double opd2,
 // (which is rounded once; the general form rounds 1/pz and its product with L),
 // and sg's change L (1 - (1 - g0)(1 + w)) = L (g0 - w + g0 w) to 2^-46 of g0 L, below
 // the 2^-53 L the float64 form's cancellation leaves.  Momenta or u beyond the
-// series (|p| >= 31 mrad) and non-finite ones take the general form; psp:
-// where psigma is when the state does not hold it.
+// series (|p| >= 31 mrad), non-finite ones and psigma without a g0 (slip) take
+// the general form; psp: where psigma is when the state does not hold it.
 //
 // Without SERIES: the general form throughout, sg's change kept as an F2 (it
 // is some 1e-3 of a metre: 2^-46 of it is below sg's rounding).
@@ -186,8 +194,9 @@ __device__ __forceinline__ void map_drift(State& s, const DevElem& e, const PsCo
     }
     const F2 u = f2_mul(f2_add(f2_sqr(c.px), f2_sqr(c.py)), c.rr);
     const uint32_t m = max(abs_hi(s.px), abs_hi(s.py));
-    if (m < 0x3fe00000u && u.h < kDriftMaxU) {
-      const F2 w = rsqrt1m_series(u), g0 = f2_unpack(k.d1), L = f2_unpack(e.p[1]);
+    const F2 g0 = f2_unpack(k.d1);
+    if (m < 0x3fe00000u && u.h < kDriftMaxU && g0.h < kNoSlip) {
+      const F2 w = rsqrt1m_series(u), L = f2_unpack(e.p[1]);
       const F2 we{w.h, f_add(w.l, k.eps)};  // d0 (1 + w + eps) = r0 (1 + w) to 2^-64
       const double Lr = fma(e.p[0], k.d0, f2_to_double(f2_mul(f2_mul(L, c.r0), we)));
       s.x = fma(Lr, s.px, s.x);
