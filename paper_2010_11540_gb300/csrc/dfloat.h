@@ -171,4 +171,15 @@ SC_HD F2 quad_slip(F2 x0, F2 px0, F2 y0, F2 py0, F2 x1, F2 px1, F2 y1, F2 py1, F
   return f2_add(f2_mul(ps, Lg), f2_neg(f2_add(f2_mul(pp, L4), f2_mul(t, qi))));
 }
 
+// The sum of the sizes of quad_slip's terms, its differences' two sides counted
+// apart: what the 14 2^-46 above are of.
+SC_HD float quad_slip_size(F2 x0, F2 px0, F2 y0, F2 py0, F2 x1, F2 px1, F2 y1, F2 py1, F2 ps, F2 qi, F2 L4, F2 Lg, F2 K) {
+  const float k = fabsf(K.h);
+  const float ax = f_fma(k, fabsf(x0.h), fabsf(px0.h)), ay = f_fma(k, fabsf(y0.h), fabsf(py0.h));
+  const float t = f_fma(fabsf(x1.h), fabsf(px1.h),
+                        f_fma(fabsf(y1.h), fabsf(py1.h), f_fma(fabsf(x0.h), ax, f_mul(fabsf(y0.h), ay))));
+  const float pp = f_fma(px0.h, px0.h, f_mul(py0.h, py0.h));
+  return f_fma(fabsf(ps.h), fabsf(Lg.h), f_fma(pp, L4.h, f_mul(t, fabsf(qi.h))));
+}
+
 }  // namespace sc

@@ -29,7 +29,20 @@ enum : int { QF_ZERO = 0, QF_FOCUS_X = 1, QF_FOCUS_Y = 2, QF_KIND = 3, QF_FAM_SH
 // sin/cos/sinh/cosh are used.
 constexpr double kMaxDelta = 0.00390625;
 
-// A g0 of the plan (PsConst) that stands for none: the drift takes its general form.
+// What may go to sg as a float pair, per length of the element.  Float64 rounds
+// 1 - (1 + beta0^2 ps)/pz, a drift's slip, by up to 7 2^-53, whatever the slip
+// itself; a pair rounds by 2^-46 of its terms some ten (drift) to fourteen
+// times (quadrupole) over, at most 3.5 2^-53 where they are below kMaxSlip.  That
+// is psigma of 3% at 3 GeV or 0.4% at 400 MeV, and some 0.1 m off axis in a
+// quadrupole; beyond, the float64 sums.  The change carried along grows by a
+// drift's while it is below kMaxCarry of its length: 2^-46 of it is 2^-53.
+// (Against no limits: one turn of 1e6 particles, 128^2, TF32 14.9 -> 15.1 ms, a
+// batch 109.5 -> 110.4.  A limit for quadrupoles relative to sg itself made a
+// sorted bunch in 32 slices 23% slower: the block that holds sg = 0 took the
+// float64 sum in nearly every warp, and the launch waited for it.)
+constexpr float kMaxSlip = 0.001953125f;
+constexpr float kMaxCarry = 0.0078125f;
+// A g0 of the plan (PsConst) that stands for none.
 constexpr float kNoSlip = 1e30f;
 
 struct State {
@@ -152,6 +165,11 @@ struct Carry {
   F2 sg;       // change of sg not yet added to the state
   bool has_sg;
 };
+__device__ __forceinline__ void carry_to_state(State& s, Carry& c) {
+  if (c.has_sg) s.sg += f2_to_double(c.sg);
+  c.sg = F2{0.f, 0.f};
+  c.has_sg = false;
+}
 
 // Exact drift (Sec. III-A): with pz = sqrt((1+delta)^2 - px^2 - py^2),
 // x += L px/pz, y += L py/pz, sg += L (1 - (1 + beta0^2 ps)/pz).
@@ -172,12 +190,12 @@ __device__ __forceinline__ double drift_general(State& s, double L, double opd2,
 // eps)) and the two sums.  w is good to 2^-54, below the rounding of L/pz
 // (which is rounded once; the general form rounds 1/pz and its product with L),
 // and sg's change L (1 - (1 - g0)(1 + w)) = L (g0 - w + g0 w) to 2^-46 of g0 L, below
-// the 2^-53 L the float64 form's cancellation leaves.  Momenta or u beyond the
-// series (|p| >= 31 mrad), non-finite ones and psigma without a g0 (slip) take
-// the general form; psp: where psigma is when the state does not hold it.
+// the 2^-53 L the float64 form's cancellation leaves (kMaxSlip).  Momenta or u beyond
+// the series (|p| >= 31 mrad), non-finite ones and psigma of a larger g0 or none
+// (slip) take the general form; psp: where psigma is when the state does not hold it.
 //
-// Without SERIES: the general form throughout, sg's change kept as an F2 (it
-// is some 1e-3 of a metre: 2^-46 of it is below sg's rounding).
+// Without SERIES: the general form throughout, sg's change carried as an F2 where
+// it is as small.
 template <bool SERIES>
 __device__ __forceinline__ void map_drift(State& s, const DevElem& e, const PsConst& k, Carry& c, const double* psp,
                                           double beta0_sq) {
@@ -195,13 +213,14 @@ __device__ __forceinline__ void map_drift(State& s, const DevElem& e, const PsCo
     const F2 u = f2_mul(f2_add(f2_sqr(c.px), f2_sqr(c.py)), c.rr);
     const uint32_t m = max(abs_hi(s.px), abs_hi(s.py));
     const F2 g0 = f2_unpack(k.d1);
-    if (m < 0x3fe00000u && u.h < kDriftMaxU && g0.h < kNoSlip) {
+    if (m < 0x3fe00000u && u.h < kDriftMaxU && fabsf(g0.h) < kMaxSlip) {
       const F2 w = rsqrt1m_series(u), L = f2_unpack(e.p[1]);
       const F2 we{w.h, f_add(w.l, k.eps)};  // d0 (1 + w + eps) = r0 (1 + w) to 2^-64
       const double Lr = fma(e.p[0], k.d0, f2_to_double(f2_mul(f2_mul(L, c.r0), we)));
       s.x = fma(Lr, s.px, s.x);
       s.y = fma(Lr, s.py, s.y);
       const F2 q = f2_add(f2_add(g0, f2_neg(w)), f2_mul(g0, w));
+      if (fabsf(c.sg.h) > kMaxCarry * L.h) carry_to_state(s, c);
       c.sg = f2_add(c.sg, f2_mul(q, L));
       c.has_sg = true;
     } else {
@@ -210,7 +229,9 @@ __device__ __forceinline__ void map_drift(State& s, const DevElem& e, const PsCo
     }
   } else {
     const double d = drift_general(s, e.p[0], k.d0, k.d1);
-    if (abs_hi(d) < kHi2p50) {
+    const double L = e.p[0];
+    if (abs_hi(d) < kHi2p50 && abs_hi(d) + (9u << 20) < abs_hi(L)) {  // 2^-9 L (kMaxSlip)
+      if (fabsf(c.sg.h) > kMaxCarry * f2_unpack(e.p[1]).h) carry_to_state(s, c);
       c.sg = f2_add(c.sg, f2_split(d));
       c.has_sg = true;
     } else {
@@ -233,7 +254,7 @@ __device__ __forceinline__ void map_drift(State& s, const DevElem& e, const PsCo
 // which gives sg += ps L/gamma0^2 - (L S2 + D) / (4 (1-ps)) with
 // S2 = (1-ps)(px0^2+py0^2) + k1 (x0^2 - y0^2), D = [x px + y py]_0^L, i.e.
 //   sg += ps L/gamma0^2 - (L/4)(px0^2+py0^2) - (L k1 (x0^2-y0^2) + D) / (4 (1-ps)),
-// in float pairs (quad_slip: some 1e-6 of a metre, good to 2^-42 of itself).
+// in float pairs (quad_slip: some 1e-6 of a metre, good to 2^-42 of itself; kMaxSlip).
 // e.p = {L/4, L/gamma0^2, cos theta0, sin theta0, cosh theta0, sinh theta0, sqk, 1/sqk, L k1,
 //        then L/4, L/gamma0^2 and L k1 as F2}
 // (theta0 = sqk L = sqk (4 e.p[0]), the host's product bit for bit), e.flags =
@@ -275,7 +296,7 @@ __device__ __forceinline__ QuadCoef quad_coef(const DevElem& e, double ps, doubl
   return QuadCoef{ch, a * sh, bq * sh, c, a * sn, -bq * sn};
 }
 
-// sg's change in float64, for states quad_slip's floats cannot hold.
+// sg's change in float64, for states quad_slip's floats cannot hold or are too short for.
 __device__ __forceinline__ void quad_slip_slow(State& s, const DevElem& e, double x0, double px0, double y0, double py0) {
   const double xy = fma(x0, x0, -y0 * y0);
   const double pp = fma(px0, px0, py0 * py0);
@@ -294,11 +315,13 @@ __device__ __forceinline__ void quad_apply(State& s, const DevElem& e, const Qua
   c.px = f2_split(s.px);
   c.py = f2_split(s.py);
   c.split = true;
-  const F2 d = quad_slip(f2_split(x0), p0, f2_split(y0), q0, f2_split(s.x), c.px, f2_split(s.y), c.py, f2_split(s.ps),
-                         k.qi, f2_unpack(e.p[9]), f2_unpack(e.p[10]), f2_unpack(e.p[11]));
+  const F2 a0 = f2_split(x0), b0 = f2_split(y0), a1 = f2_split(s.x), b1 = f2_split(s.y), ps = f2_split(s.ps);
+  const F2 L4 = f2_unpack(e.p[9]), Lg = f2_unpack(e.p[10]), K = f2_unpack(e.p[11]);
+  const float size = quad_slip_size(a0, p0, b0, q0, a1, c.px, b1, c.py, ps, k.qi, L4, Lg, K);
+  const F2 d = quad_slip(a0, p0, b0, q0, a1, c.px, b1, c.py, ps, k.qi, L4, Lg, K);
   const uint32_t m = max(max(max(abs_hi(x0), abs_hi(px0)), max(abs_hi(y0), abs_hi(py0))),
                          max(max(abs_hi(s.x), abs_hi(s.px)), max(max(abs_hi(s.y), abs_hi(s.py)), abs_hi(s.ps))));
-  if (m < kHi2p50 && fabsf(d.h) < 1e30f) {
+  if (m < kHi2p50 && size < 4.f * kMaxSlip * L4.h) {  // (L4 = L/4)
     c.sg = f2_add(c.sg, d);
     c.has_sg = true;
   } else {
@@ -466,9 +489,8 @@ __device__ __forceinline__ bool push_elements(State& s, PsConst& k, const DevEle
         c.split = false;
         break;
       case SC_RF:
-        if (c.has_sg) s.sg += f2_to_double(c.sg);  // the cavity reads sg
-        c.sg = F2{0.f, 0.f};
-        c.has_sg = c.has_rr = false;
+        carry_to_state(s, c);  // the cavity reads sg
+        c.has_rr = false;
         map_rf(s, e);
         ps_const<SERIES, WIDE, true>(k, s.ps, beta0_sq, quads);
         changed = true;
