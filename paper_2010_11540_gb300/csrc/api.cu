@@ -437,6 +437,7 @@ sc_status create_grid(sc_grid** out, int nx, int ny, double xmin, double xmax, d
   g->geom.ay = make_fix_axis(ymin, g->geom.inv_hy, ny - 1);
   if (n_slices > 1) g->geom.az = make_fix_axis(zmin, g->geom.inv_dz, n_slices);
   g->geom.fix = g->geom.ax.top && g->geom.ay.top && (n_slices == 1 || g->geom.az.top);
+  if (g->geom.fix && fix_fraction_serves(g->geom.ax) && fix_fraction_serves(g->geom.ay)) g->geom.fix = 2;
   g->sum_axes.x = make_sum_axis(xmin, g->geom.inv_hx, nx - 1);
   g->sum_axes.y = make_sum_axis(ymin, g->geom.inv_hy, ny - 1);
   if (n_slices > 1) g->sum_axes.z = make_sum_axis(zmin, g->geom.inv_dz, n_slices);

@@ -36,12 +36,11 @@ __device__ __noinline__ int locate_exact(const GridGeom& g, double x, double y, 
 // took 4 of its instructions per particle, 6 on sliced grids, 64 clocks each):
 // for the one particle in some millions that lies too near a place where the
 // decision changes, and on axes the integers do not serve (GridGeom::fix),
-// locate_exact decides.  (Stand-alone deposit of 1e6 particles 11.7 -> 10.1 us,
-// 1e7 in 32 slices 130 -> 107 us; one turn of 4e6 particles, BF16, 71.4 -> 64.5 ms.)
+// locate_exact decides.  (One turn of 4e6 particles, BF16, 71.4 -> 64.5 ms.)
 template <bool FRAC>
 __device__ __forceinline__ int locate(const GridGeom& g, double x, double y, double sg, int2& a, double& fx,
                                       double& fy, int& i, int& j, int& k) {
-  if (g.fix) {
+  if (FRAC ? g.fix > 1 : g.fix != 0) {
     uint64_t zx, zy, zz;
     k = 0;
     int in = fix_split(g.ax, x, i, a.x, zx);

@@ -219,6 +219,14 @@ SC_HD double fix_fraction(const FixAxis& a, uint64_t z) {
   return bits_f64(((uint64_t)(1021 - n) << 52) + ((fr << n) >> 11));  // the leading bit adds one to the exponent
 }
 
+// Whether those fractions are as good as the two-rounding ones, which are off
+// by up to cells 2^-53 in mid-grid: four units of 2^-F (x, xmin and the product
+// truncated, T's place) no larger.  Not so on grids more than some thirty of
+// their widths off centre.
+inline bool fix_fraction_serves(const FixAxis& a) {
+  return a.top && (((unsigned __int128)a.limit << a.f) >> 55) != 0;
+}
+
 // The leading 64 bits of a b from three 32 x 32-bit products, short by at most three units.
 SC_HD uint64_t mulhi64_near(uint64_t a, uint64_t b) {
   const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;

@@ -70,7 +70,7 @@ struct GridGeom {
   // slice, held in a block's shared memory (the whole slice when it fits in
   // kTileBytes, else the centred window that does)
   int wx0, wy0, wnx, wny;
-  // the axes in integers (x, y, and sigma when sliced); fix: all of them usable
+  // the axes in integers (x, y, and sigma when sliced); fix: 1 all of them usable, 2 for float64 fractions too
   FixAxis ax, ay, az;
   int fix;
 };
