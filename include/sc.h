@@ -358,6 +358,10 @@ sc_status sc_set_solver_tiling(sc_grid *g, const int *choice);
  * sc_set_kick_push_shape fixes either part (the next sc_track_turns
  * re-captures); sc_get_kick_push_shape reads the shape of the captured turn
  * and, in trial_us, the timed trial of the chosen shape (0 when not timed).
+ * A block size neither fixed nor timed (trial_us 0 and none set) reads as the
+ * largest: the launches of such a turn take that or, each by the bunch's size
+ * and its own deposit tile, 384 threads; fixing the value read makes all of
+ * them take it (the same bits in another time).
  * Errors: SC_ERR_ARG (NULL grid, a value out of range, or no captured turn). */
 sc_status sc_set_kick_push_shape(sc_grid *g, int threads, int traversal);
 sc_status sc_get_kick_push_shape(sc_grid *g, int *threads, int *traversal, double *trial_us);

@@ -388,7 +388,9 @@ def set_kick_push_shape(grid: Grid, threads: int = 0, traversal: int = -1):
 
 def get_kick_push_shape(grid: Grid):
     """-> (threads, traversal, trial_us) of the grid's captured turn (trial_us:
-    the timed trial of the chosen shape, 0 when the shape was not timed)."""
+    the timed trial of the chosen shape, 0 when the shape was not timed).
+    threads neither fixed nor timed reads as the largest; small bunches'
+    launches may then take 384 (include/sc.h)."""
     t, v, us = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_double(0)
     _check(load().sc_get_kick_push_shape(grid.handle, ctypes.byref(t), ctypes.byref(v), ctypes.byref(us)))
     return int(t.value), int(v.value), us.value
