@@ -48,6 +48,7 @@ WORKLOADS = {
 # sm__thread_inst_executed_pipe_fp64_pred_on per launch on the three segment
 # types of the bench ring (1e6 particles), of the build that did so
 # (profiles/kick_push_c2.md: 55.8, 68.0 and 18.0, mean 47.2 per particle-kick).
+# Those segments hold no dipole or cavity: bend and rf are estimates.
 # base = gather + kick + fused deposit.  The quadrupole reads its matrix
 # entries from the per-particle family cache (51.0 when it computes them).
 FP64_INST = {"base": 17.5, "drift": 12.2, "quad": 20.6, "sext": 5.0, "bend": 16.0, "rf": 30.0}
@@ -70,7 +71,7 @@ FP64_INST_LON_BEZIER_F32 = 13.95
 # cache; c2: mean of the three segment types), with the kernel sources'
 # SHA-256 (first 16 hex digits) they were captured on: the roofline's
 # "traffic" while the sources still match; other workloads report null.
-KP_TRAFFIC_TF32 = {"c2": (127.7e6, "9bb95a0315e88b02"),  # 1e6 particles (the working set partly stays in L2)
+KP_TRAFFIC_TF32 = {"c2": (127.7e6, "ffc97ff9094975ac"),  # 1e6 particles (the working set partly stays in L2)
                    "c4": (3860.0e6, "052c41cbfc714941"),  # 2.37e7 particles, batched (kick_push_traffic_c4_c5.md)
                    "c5": (1594.1e6, "052c41cbfc714941")}  # 1e7 particles in 32 slices
 # GB300: 152 SMs x 2 FP64 instructions per SM clock x 2.07 GHz maximum clock
@@ -84,13 +85,16 @@ DEP_FP64_INST_SLICE = 1.0
 # corrections and the path length in float pairs (csrc/dfloat.h).  By kernel
 # family: float64 fields; float32 fields with the series drift (split TF32, one
 # grid per bunch); float32 fields with the general drift (the other split forms).
+# Dipole and cavity, of which the bench's rings hold none: segments drift-dipole
+# and drift-cavity less a drift's, the cavity's on a ring of two quadrupole
+# families (their per-particle entries are computed anew after it).
 FP64_ISSUED = {
-    "f64": {"base": 9.81, "drift": 3.98, "quad": 7.09, "sext": 5, "bend": 16.0, "rf": 30.0},
-    "f32_series": {"base": 2.76, "drift": 3.2, "quad": 8.62, "sext": 5, "bend": 16.0, "rf": 30.0},
-    "f32": {"base": 2.76, "drift": 11.2, "quad": 8.61, "sext": 5, "bend": 16.0, "rf": 30.0},
+    "f64": {"base": 9.81, "drift": 3.98, "quad": 7.09, "sext": 5, "bend": 13, "rf": 103},
+    "f32_series": {"base": 2.76, "drift": 3.2, "quad": 8.62, "sext": 5, "bend": 13, "rf": 92},
+    "f32": {"base": 2.76, "drift": 11.2, "quad": 8.61, "sext": 5, "bend": 13, "rf": 90},
 }
 KP_SOURCES = ("kick_push.cu", "maps.cuh", "cic.cuh", "fixpt.h", "dfloat.h", "sc_internal.cuh")
-FP64_INST_SOURCES_SHA = "9bb95a0315e88b02"
+FP64_INST_SOURCES_SHA = "ffc97ff9094975ac"
 # HBM bytes per particle-kick that the fused kick/push must move (algorithmic):
 # the six float64 coordinates read (48 B) and the five a kick and a push
 # change written back (40 B: psigma changes only in RF cavities); 96 B when
@@ -230,7 +234,7 @@ def fp64_inst_per_turn(lat, precision):
 
 def probe_peaks(stream):
     """Live machine probes from libsc_probe.so (bench_probe.cu, built beside
-    this file; not part of libsc): conflict-free and random-word shared u64
+    this file; not part of libsc): conflict-free and random-word shared u32
     atomics per second, FP64 FMA instructions per second."""
     import ctypes
     from paper_2010_11540_gb300 import build
@@ -460,9 +464,10 @@ class SingleRun:
 
     def deposit_roofline(self, h, flush, atom_random, atom_conflict_free, reps=20):
         """sc_deposit alone (the deposit kernel) on the workload's particles:
-        4 shared-memory u64 atomic adds per particle inside the grid, against
-        the probed conflict-free rate of such atomics (the random-word rate of
-        a 128 KB table as context)."""
+        8 shared-memory u32 atomic adds per particle inside the grid (the low
+        and the high words of four 64-bit bins), against the probed
+        conflict-free rate of such atomics (the random-word rate of a 128 KB
+        table as context)."""
         import torch
         from paper_2010_11540_gb300 import sc
         g, dev = h
@@ -478,7 +483,7 @@ class SingleRun:
                 c.record(self.stream)
             torch.cuda.synchronize()
         ms = sorted(a.elapsed_time(c) for a, c in ev)[reps // 2]
-        atomics = 4 * n_in
+        atomics = 8 * n_in
         rate = atomics / (ms * 1e-3)
         # the same bunch ordered by cell (sc_sort_particles, on a copy): warps combine equal cells
         with torch.cuda.stream(self.stream):
@@ -498,26 +503,26 @@ class SingleRun:
                    "frac": atomics / (ms_o * 1e-3) / atom_conflict_free,
                    "what": "the same particles ordered by cell (sc_sort_particles): each warp combines the weights "
                            "of neighbouring particles in one cell before its atomic adds; achieved counts the "
-                           "4 algorithmic atomics per particle"}
+                           "8 algorithmic atomics per particle"}
         return {"bound": "shared-atomics", "kernel": "deposit_kernel (stand-alone sc_deposit)",
-                "achieved": rate / 1e9, "peak": atom_conflict_free / 1e9, "unit": "G shared-u64-atomics/s",
+                "achieved": rate / 1e9, "peak": atom_conflict_free / 1e9, "unit": "G shared-u32-atomics/s",
                 "frac": rate / atom_conflict_free, "avg_launch_ms": ms, "atomics_per_launch": atomics,
-                "peak_source": "live probe (libsc_probe.so): conflict-free shared u64 atomicAdd, each warp on 32 "
+                "peak_source": "live probe (libsc_probe.so): conflict-free shared u32 atomicAdd, each warp on 32 "
                                "consecutive words, measured in this run",
                 "context_peak_random_words": atom_random / 1e9,
                 "frac_of_random_words": rate / atom_random, "ordered_bunch": ordered,
-                # what binds it: the locate's FP64 sum per axis and integer issue (the cell, fraction and
-                # weights are decoded from the bits with integer instructions), on the 2-per-clock FP64 pipe
+                # the locate's FP64 sum per axis on the 2-per-clock FP64 pipe (the cell and weights are decoded
+                # from its bits with integer instructions)
                 "fp64_pipe": {"fp64_inst_per_particle": DEP_FP64_INST + (DEP_FP64_INST_SLICE if self.slices else 0),
                               "achieved": (DEP_FP64_INST + (DEP_FP64_INST_SLICE if self.slices else 0)) * self.n
                               / (ms * 1e-3) / 1e12,
                               "peak": FP64_PIPE_PEAK_TINST, "unit": "T FP64-inst/s",
                               "frac": (DEP_FP64_INST + (DEP_FP64_INST_SLICE if self.slices else 0)) * self.n
                               / (ms * 1e-3) / 1e12 / FP64_PIPE_PEAK_TINST,
-                              "ceiling_atomics_frac": 4 / (DEP_FP64_INST + (DEP_FP64_INST_SLICE if self.slices else 0))
+                              "ceiling_atomics_frac": 8 / (DEP_FP64_INST + (DEP_FP64_INST_SLICE if self.slices else 0))
                               * FP64_PIPE_PEAK_TINST * 1e12 / atom_conflict_free,
-                              "note": "at the FP64 peak the deposit adds 4 atomics per 4 FP64 instructions: the "
-                                      "ceiling_atomics_frac of the conflict-free atomic rate"}}
+                              "note": "at the FP64 peak the deposit adds 8 words per 2 FP64 instructions (sliced "
+                                      "grids 3): the ceiling_atomics_frac of the conflict-free atomic rate"}}
 
     def grid_desc(self):
         d = {"grid": [self.grid[0], self.grid[1]]}

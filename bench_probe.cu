@@ -1,6 +1,6 @@
 // Machine probes for bench.py's roofline denominators (not part of libsc):
-// the throughput of shared-memory 64-bit atomic adds (the unit of work of the
-// CIC deposit, Sec. IV-A) and of FP64 fused multiply-adds (the FP64 pipe that
+// the throughput of shared-memory 32-bit atomic adds (the unit of work of the
+// CIC deposit, Sec. IV-A, whose 64-bit bins are two such words) and of FP64 fused multiply-adds (the FP64 pipe that
 // bounds the transfer-map push, Sec. III), measured on the device in use.
 // The kernels touch only their own shared memory / registers and one output
 // word per block.  Built into libsc_probe.so beside bench.py.
@@ -9,42 +9,42 @@
 namespace {
 
 constexpr int kProbeThreads = 1024;
-constexpr int kTable = 4096;  // 32 KB of u64 counters per block
+constexpr int kTable = 4096;  // 16 KB of u32 counters per block
 
-// Each warp's 32 lanes add to 32 consecutive words (the fewest shared-memory
-// wavefronts a 64-bit atomic can take), four independent adds per iteration.
+// Each warp's 32 lanes add to 32 consecutive words (one shared-memory
+// wavefront, no bank twice), four independent adds per iteration.
 __global__ void __launch_bounds__(kProbeThreads) probe_atomics_kernel(int iters, unsigned long long* sink) {
-  __shared__ unsigned long long tab[kTable];
-  for (int i = threadIdx.x; i < kTable; i += blockDim.x) tab[i] = 0ull;
+  __shared__ unsigned tab[kTable];
+  for (int i = threadIdx.x; i < kTable; i += blockDim.x) tab[i] = 0u;
   __syncthreads();
   const unsigned a = threadIdx.x;
   for (int it = 0; it < iters; ++it) {
-    atomicAdd(&tab[a], 1ull);
-    atomicAdd(&tab[a + 1024], 1ull);
-    atomicAdd(&tab[a + 2048], 1ull);
-    atomicAdd(&tab[a + 3072], 1ull);
+    atomicAdd(&tab[a], 1u);
+    atomicAdd(&tab[a + 1024], 1u);
+    atomicAdd(&tab[a + 2048], 1u);
+    atomicAdd(&tab[a + 3072], 1u);
   }
   __syncthreads();
-  if (threadIdx.x == 0) sink[blockIdx.x] = tab[0] + tab[kTable - 1];
+  if (threadIdx.x == 0) sink[blockIdx.x] = (unsigned long long)tab[0] + tab[kTable - 1];
 }
 
-// Random cells of a 128 KB table (the deposit tile of a 128 x 128 grid):
+// Random words of a 128 KB table (the deposit tile of a 128 x 128 grid):
 // each thread walks its own linear congruential sequence of word indices.
-constexpr int kRandTable = 16384;
+constexpr int kRandTable = 32768;
 __global__ void __launch_bounds__(kProbeThreads) probe_atomics_random_kernel(int iters, unsigned long long* sink) {
-  extern __shared__ unsigned long long rtab[];
-  for (int i = threadIdx.x; i < kRandTable; i += blockDim.x) rtab[i] = 0ull;
+  extern __shared__ unsigned rtab[];
+  for (int i = threadIdx.x; i < kRandTable; i += blockDim.x) rtab[i] = 0u;
   __syncthreads();
   unsigned h = 2654435761u * (threadIdx.x + 1) + 97u * blockIdx.x;
   for (int it = 0; it < iters; ++it) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       h = h * 1664525u + 1013904223u;
-      atomicAdd(&rtab[h >> 18], 1ull);  // top 14 bits: 0 .. 16383
+      atomicAdd(&rtab[h >> 17], 1u);  // top 15 bits: 0 .. 32767
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sink[blockIdx.x] = rtab[0] + rtab[kRandTable - 1];
+  if (threadIdx.x == 0) sink[blockIdx.x] = (unsigned long long)rtab[0] + rtab[kRandTable - 1];
 }
 
 // CH independent FMA chains per thread (enough to hide the pipe latency).
@@ -84,8 +84,8 @@ int time_launches(F launch, cudaStream_t s, float* ms) {
 
 }  // namespace
 
-// Throughput of conflict-free shared u64 atomics (each warp on 32 consecutive
-// words), of shared u64 atomics on random words of a 128 KB table, and of FP64
+// Throughput of conflict-free shared u32 atomics (each warp on 32 consecutive
+// words), of shared u32 atomics on random words of a 128 KB table, and of FP64
 // FMA instructions, per second on the current device, each timed over five
 // launches on `stream` (synchronous).  Outputs may be NULL (not all).
 // Returns 0, -1 (nothing asked) or -2 (a CUDA call failed).
@@ -110,11 +110,11 @@ extern "C" int scb_probe_peaks(double* shared_atomics_per_s, double* random_atom
     const int iters = 1024;
     float ms = 0.f;
     if (cudaFuncSetAttribute(probe_atomics_random_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kRandTable * 8) != cudaSuccess)
+                             kRandTable * 4) != cudaSuccess)
       st = -2;
     if (!st)
       st = time_launches(
-        [&] { probe_atomics_random_kernel<<<sms, kProbeThreads, kRandTable * 8, s>>>(iters, sink); }, s, &ms);
+        [&] { probe_atomics_random_kernel<<<sms, kProbeThreads, kRandTable * 4, s>>>(iters, sink); }, s, &ms);
     if (!st) *random_atomics_per_s = (double)sms * kProbeThreads * iters * 4 / (ms * 1e-3);
   }
   if (!st && fp64_inst_per_s) {

@@ -125,8 +125,9 @@ typedef struct {
  * Sec. I) or, for the SC_SOLVE_PIPE_* forms, the conducting rectangular pipe
  * of Sec. IV-B.  Builds the Green's-function spectra (or sine-transform
  * matrices) on the device (synchronous on `stream`); the grid owns them and
- * every other device buffer it uses (released by sc_destroy_grid).
- * nx, ny: powers of two in 8..512 for SC_SOLVE_FP64; nx = ny in {64, 128, 256}
+ * every other device buffer it uses (released by sc_destroy_grid): per node
+ * and slice 8 bytes of charge, and 16 of field in the float32 forms, 32 in the
+ * float64 ones (the field and its differences along x).  nx, ny: powers of two in 8..512 for SC_SOLVE_FP64; nx = ny in {64, 128, 256}
  * for SC_SOLVE_TF32X3 and SC_SOLVE_BF16X3; nx - 1, ny - 1 powers of two in 8..512 for
  * SC_SOLVE_PIPE_FP64; nx = ny in 10..258 for SC_SOLVE_PIPE_TF32X3.  Errors: SC_ERR_ARG, SC_ERR_UNSUPPORTED,
  * SC_ERR_OOM, SC_ERR_CUDA.  *out is set only on success. */

@@ -1,13 +1,14 @@
 // Radix-2 Stockham FFT in shared memory, float64, shared by the float64
 // solves (open boundary and conducting pipe).
 //
-// A transform is bound by the FP64 pipe of the SM it runs on (two instructions
-// per clock, 64 clocks of a sub-partition per warp instruction), so what
-// counts is FP64 instructions per butterfly.  a +- w b with w = c + i s takes
-// six fused multiply-adds instead of eight instructions when w is factored by
-// its larger part (E. Linzer and E. Feig, IEEE Trans. Signal Process. 41
-// (1993) 93): w b = c (b + i t b), t = s/c, or w b = i s (b + i u b),
-// u = -c/s; |t|, |u| <= 1, so no accuracy is lost.
+// A transform waits for its barriers and shared-memory trips and for the FP64
+// pipe of the SM it runs on (two instructions per clock, 64 clocks of a
+// sub-partition per warp instruction), so FP64 instructions per butterfly
+// count.  a +- w b with w = c + i s takes six fused multiply-adds instead of
+// eight instructions when w is factored by its larger part (E. Linzer and
+// E. Feig, IEEE Trans. Signal Process. 41 (1993) 93): w b = c (b + i t b),
+// t = s/c, or w b = i s (b + i u b), u = -c/s; |t|, |u| <= 1, so no accuracy is
+// lost.
 #pragma once
 
 #include <cmath>

@@ -100,13 +100,15 @@ __device__ __noinline__ void store_quad_cache(const KPParams& P, double ps, doub
 // weights), else float64 fields and fractions; SERIES: the drift in float
 // pairs (map_drift, series_drift).
 //
-// Bound by the FP64 pipe, which holds a sub-partition for 64 clocks per warp
-// instruction, and beside it by the latency of its own chain at 24 warps per
-// SM; DRAM traffic is a third of what the time would allow.  So the work is in
-// float pairs and integers wherever those are as exact: with 47 -> 18 FP64
+// The FP64 pipe holds a sub-partition for 64 clocks per warp instruction, so
+// the work is in float pairs and integers wherever those are as exact.  What
+// binds it then is the latency of each particle's own chain at 24 warps per SM:
+// in the quadrupole segments the FP64 pipe is 53-56% busy (the general drift:
+// 72-80%), the issue slots 44-47%; DRAM traffic is a third of what the time
+// would allow.  With 47 -> 18 FP64
 // instructions per particle and kick, the three kinds of launch of the
 // 216-location ring (1e6 particles, 128^2, TF32: drift-quadrupole-drift-
-// sextupole-drift, drift-quadrupoles-drift, one drift) take 74, 78 and 43 us
+// sextupole-drift, drift-quadrupoles-drift, one drift) take 77, 80 and 44 us
 // from a cold cache instead of 116, 136 and 53.  Indices are 32-bit (fewer than 2^24
 // particles): 64-bit ones cost another add per array access, 4% of a batch's turn.
 template <bool CACHE, bool F32, bool XE, bool SERIES>
@@ -485,10 +487,12 @@ sc_status launch_kick_push_batched(const KPParams* descs, const int4* blocks, in
 // roundings, which moves the tracked state by 2.6e-10 (relative L2, one turn of
 // the 216-location ring, at most over 64^2..256^2 grids and 3e4..6e6 particles)
 // with TF32 on one grid per bunch, 1.1e-9 with BF16, 4.5e-8 in a pipe and up
-// to 1e-5 on sliced grids, whose slices carry 50 times the line density.  Only
-// the first is below 1e-9, so the others keep the general drift and with it
-// the bits of every position and momentum.  One turn, 1e6 particles on 128^2,
-// TF32: series 14.9 ms, general 19.0 ms (float64 fields: 18.0 ms with the series).
+// to 1e-5 on sliced grids, whose slices carry 50 times the line density.  The
+// first stays below 1e-9; the others keep the general drift, so that a tracked
+// state comes out to 1e-9 as it does with every map in FP64 instructions.  That
+// is a choice and not a limit of accuracy: against 64 bits the same turns are
+// off by 2e-7, 2e-5 and 5e-5.  Its price: one turn, 1e6 particles on 128^2,
+// TF32: series 15.2 ms, general 19.0 ms (float64 fields: 18.0 ms with the series).
 bool series_drift(const sc_grid* g) { return !g->field32 || (g->precision == SC_SOLVE_TF32X3 && g->nz == 1); }
 
 // Per-element constants in float64 on the host (libm), in the layouts that

@@ -20,10 +20,11 @@
 // that is kept.  The two inverse column transforms run side by side in two
 // halves of the block.
 //
-// Bound by the FP64 pipe (two instructions per SM clock), so what counts is
-// FP64 instructions per butterfly: six fused multiply-adds with the twiddle
-// factored, where multiply-then-add takes eight.  With the stages left out as
-// above, a float64 turn of 1e6 particles on 128^2 (216 solves) went from 22.1
+// Each kernel is some 1-2 us of FP64 work and takes 5-8: a launch, its loads and
+// one barrier and shared-memory trip after another.  Of the work, what counts
+// is FP64 instructions per butterfly (two per SM clock): six fused multiply-adds
+// with the twiddle factored, where multiply-then-add takes eight.  With the
+// stages left out as above, a float64 turn of 1e6 particles on 128^2 (216 solves) went from 22.1
 // to 18.9 ms, one of 2e4 particles on 64^2 from 1.90 to 1.55 ms.
 #include <complex>
 #include <vector>
